@@ -1259,53 +1259,121 @@ __device__ __forceinline__ void merge_phase(const FrameArgs& a) {
     }
 }
 
-// Root of a label whose parent has already been loaded (no union runs any more; L2 loads, as
-// other threads overwrite labels with roots meanwhile -- an ancestor either way).
-__device__ __forceinline__ int root_from(const int32_t* L, int x, int p) {
-    while (p != x) {
-        x = p;
-        p = __ldcg(L + x);
+// Flatten: every grouped triangle takes its root, in blocks of kFlatBlock consecutive labels per
+// warp, kFlatVec 16-byte loads per lane. A triangle's label is the root of its tile's segment, whose
+// parent chain (one or two hops, measured) ends at the segment's root.
+//
+// What bounds it: most of a frame's chains end at a few roots (the floor, a wall), so thousands of
+// warps ask for the same words. Read past L1 those requests queue at one L2 slice: on a batch of 256
+// mixed frames (73.9 M triangles) the mean warp took 0.6 ms and the last one 1.9 ms. The parents are
+// therefore read through L1: the grid barrier before this phase acquires at GPU scope, so a line
+// cached here is no older than the last union, and a word that another thread has meanwhile replaced
+// by its root was and is an ancestor, either way. The labels themselves are read once, past L1, 16
+// bytes per lane. With both, the phase took 0.38 ms and the batch 5.88 instead of 7.40 ms; a 480x640
+// frame 69.6 instead of 73.7 us.
+constexpr int kFlatVec = 2;
+constexpr int kFlatBlock = 32 * 4 * kFlatVec;
+
+// Blocks of a frame of n labels; blocks start at 16-byte boundaries, up to 3 labels before the first.
+__device__ __forceinline__ long long flatten_blocks(long long n) { return (n + 3 + kFlatBlock - 1) / kFlatBlock; }
+
+// Block b of the labels L[0 .. n): roots into L and, when given, into `copy`; with `sizes` the
+// segment sizes are counted (an atomic per root and warp load, one per block when it has one root).
+// Called by whole warps.
+__device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* sizes, int32_t* copy, long long b) {
+    const int lane = threadIdx.x & 31;
+    const int shift = (int)(((uintptr_t)L >> 2) & 3u);
+    const long long i0 = b * kFlatBlock - shift + 4 * lane;
+    int x[4 * kFlatVec], p[4 * kFlatVec];
+    bool whole[kFlatVec];
+#pragma unroll
+    for (int v = 0; v < kFlatVec; ++v) {
+        const long long i = i0 + 128 * v;
+        whole[v] = i >= 0 && i + 4 <= n;
+        if (whole[v]) {
+            const int4 q = __ldcg(reinterpret_cast<const int4*>(L + i));
+            x[4 * v] = q.x, x[4 * v + 1] = q.y, x[4 * v + 2] = q.z, x[4 * v + 3] = q.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[4 * v + k] = i + k >= 0 && i + k < n ? __ldcg(L + i + k) : -1;
+        }
     }
-    return x;
+#pragma unroll
+    for (int k = 0; k < 4 * kFlatVec; ++k) p[k] = x[k] >= 0 ? __ldca(L + x[k]) : -1;
+    // one hop of every unfinished walk per round, their loads together
+    bool more;
+    do {
+        more = false;
+#pragma unroll
+        for (int k = 0; k < 4 * kFlatVec; ++k)
+            if (p[k] != x[k]) {
+                x[k] = p[k];
+                p[k] = __ldca(L + x[k]);
+                more = true;
+            }
+    } while (more);
+#pragma unroll
+    for (int v = 0; v < kFlatVec; ++v) {
+        const long long i = i0 + 128 * v;
+        if (whole[v]) {
+            *reinterpret_cast<int4*>(L + i) = make_int4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i + k >= 0 && i + k < n) L[i + k] = x[4 * v + k];
+        }
+        if (copy) {
+            // page-locked host memory as a rule: whole lines when it is aligned as L is (4-byte stores
+            // of every fourth word cost a 240x320 host-buffer call 3 us)
+            if (whole[v] && (((uintptr_t)copy ^ (uintptr_t)L) & 15u) == 0) {
+                *reinterpret_cast<int4*>(copy + i) = make_int4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (i + k >= 0 && i + k < n) copy[i + k] = x[4 * v + k];
+            }
+        }
+    }
+    if (sizes) {
+        __syncwarp();
+        // the block's first root; a block that has no other needs one atomic
+        int first = -1, mine = 0;
+        bool one = true;
+#pragma unroll
+        for (int k = 0; k < 4 * kFlatVec; ++k) {
+            if (x[k] < 0) continue;
+            if (first < 0) first = x[k];
+            one &= x[k] == first;
+            ++mine;
+        }
+        const unsigned have = __ballot_sync(0xffffffffu, mine > 0);
+        if (!have) return;
+        const int lead = __ffs(have) - 1;
+        const int root = __shfl_sync(0xffffffffu, first, lead);
+        if (__all_sync(0xffffffffu, mine == 0 || (one && first == root))) {
+            const int count = __reduce_add_sync(0xffffffffu, mine);
+            if (lane == lead) atomicAdd(sizes + root, count);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4 * kFlatVec; ++k) {
+                const unsigned peers = __match_any_sync(0xffffffffu, x[k]);
+                if (x[k] >= 0 && lane == __ffs(peers) - 1) atomicAdd(sizes + x[k], __popc(peers));
+            }
+        }
+    }
 }
 
-// Every grouped triangle takes its root; with tri_min > 0 the segment sizes are counted, one
-// atomic per run of equal roots in a warp. Four triangles per thread are in flight at once:
-// their labels, then their parents, are loaded together before any walk continues.
 __device__ __forceinline__ void flatten_phase(const FrameArgs& a) {
-    constexpr int U = 4;
     const long long n = 2LL * (a.H - 1) * (a.W - 1);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const long long n_iter = (n + stride - 1) / stride;   // uniform: whole warps stay together
-    const long long base = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    int32_t* L = a.labels;
+    int32_t* const L = a.labels;
     int32_t* const sizes = a.sizes;
     int32_t* const copy = sizes ? nullptr : a.labels_copy;   // with tri_min the filter writes it
-    for (long long it0 = 0; it0 < n_iter; it0 += U) {
-        int lab[U], par[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const long long i = base + (it0 + u) * stride;
-            lab[u] = (it0 + u < n_iter && i < n) ? __ldcg(L + i) : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) par[u] = lab[u] >= 0 ? __ldcg(L + lab[u]) : -1;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const long long i = base + (it0 + u) * stride;
-            int root = -1;
-            if (lab[u] >= 0) {
-                root = root_from(L, lab[u], par[u]);
-                L[i] = root;
-            }
-            if (copy && it0 + u < n_iter && i < n) copy[i] = root;
-            if (sizes) {
-                const unsigned peers = __match_any_sync(0xffffffffu, root);
-                const int leader = __ffs(peers) - 1;
-                if (root >= 0 && (int)(threadIdx.x & 31) == leader) atomicAdd(sizes + root, __popc(peers));
-            }
-        }
-    }
+    const long long blocks = flatten_blocks(n);
+    const int warps = gridDim.x * (kThreads / 32);
+    // warp k of every CTA takes blocks k gridDim.x + the CTA's index: a frame of fewer blocks than
+    // warps spreads over all SMs
+    for (long long b = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; b < blocks; b += warps)
+        flatten_block(L, n, sizes, copy, b);
 }
 
 // Algorithm 5 keeps a segment only when it has more than tri_min triangles.
@@ -1561,49 +1629,17 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
     grid_barrier(b.barrier, b.error);
     mark(2);
     {
-        // every grouped triangle takes its root; segment sizes are counted per (frame, root);
-        // four triangles per thread in flight at once, as in the single-frame flatten
-        constexpr int U = 4;
-        const long long total = __ldg(b.tris + n);
-        const long long n_iter = (total + stride - 1) / stride;   // uniform: whole warps stay together
+        // every grouped triangle takes its root, block by block. Frame f's blocks start at
+        // tris[f] / kFlatBlock + 2 f: at least flatten_blocks() of them, the last ones empty
+        const long long total = __ldg(b.tris + n) / frame::kFlatBlock + 2LL * n;
         int f = 0;
-        for (long long it0 = 0; it0 < n_iter; it0 += U) {
-            int lab[U], par[U], fr[U];
-            int32_t* lp[U];
-            long long li[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long i = base + (it0 + u) * stride;
-                lab[u] = -1;
-                fr[u] = 0;
-                lp[u] = nullptr;
-                li[u] = 0;
-                if (it0 + u < n_iter && i < total) {
-                    f = frame::advance_frame(b.tris, f, i);
-                    fr[u] = f;
-                    lp[u] = b.frames[f].labels;
-                    li[u] = i - __ldg(b.tris + f);
-                    lab[u] = __ldcg(lp[u] + li[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) par[u] = lab[u] >= 0 ? __ldcg(lp[u] + lab[u]) : -1;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                int root = -1;
-                long long key = -1;
-                if (lab[u] >= 0) {
-                    root = frame::root_from(lp[u], lab[u], par[u]);
-                    lp[u][li[u]] = root;
-                    key = ((long long)fr[u] << 32) | (unsigned)root;
-                }
-                if (any_filter) {
-                    const unsigned peers = __match_any_sync(0xffffffffu, key);
-                    const int leader = __ffs(peers) - 1;
-                    int32_t* sizes = root >= 0 ? b.frames[fr[u]].sizes : nullptr;
-                    if (sizes && (int)(threadIdx.x & 31) == leader) atomicAdd(sizes + root, __popc(peers));
-                }
-            }
+        for (long long k = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; k < total;
+             k += (long long)gridDim.x * (kThreads / 32)) {
+            while (__ldg(b.tris + f + 1) / frame::kFlatBlock + 2LL * (f + 1) <= k) ++f;
+            const long long t0 = __ldg(b.tris + f);
+            const FrameArgs& a = b.frames[f];
+            frame::flatten_block(a.labels, __ldg(b.tris + f + 1) - t0, a.sizes, nullptr,
+                                 k - (t0 / frame::kFlatBlock + 2LL * f));
         }
     }
     if (any_filter) {
