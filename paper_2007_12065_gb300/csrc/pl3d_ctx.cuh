@@ -152,8 +152,10 @@ inline void record_stop(pl3d_ctx* c, cudaStream_t s, int slot, cudaEvent_t e0, c
     c->pending.push_back({slot, e0, e1});
 }
 
-// Frees and reallocates `*ptr` to hold `need` units of `elem_per` elements (plus headroom).
-// Waits for the stream first, since work in flight may still use the old buffer.
+// Frees and reallocates `*ptr` to hold `need` units of `elem_per` elements (plus headroom, and a
+// multiple of 4 units: a buffer's second half, at 3 capacity floats, then starts 16-byte aligned like
+// the first, as the float4 stores of a second Laplacian pass need). Waits for the stream first, since
+// work in flight may still use the old buffer.
 template <class T>
 int grow(T** ptr, size_t* cap, size_t need, size_t elem_per, cudaStream_t s) {
     if (*cap >= need) return PL3D_OK;
@@ -163,7 +165,7 @@ int grow(T** ptr, size_t* cap, size_t need, size_t elem_per, cudaStream_t s) {
         *ptr = nullptr;
         *cap = 0;
     }
-    const size_t n = need + need / 8;
+    const size_t n = (need + need / 8 + 3) / 4 * 4;
     if (cudaMalloc((void**)ptr, n * elem_per * sizeof(T)) != cudaSuccess) {
         cudaGetLastError();
         *ptr = nullptr;
