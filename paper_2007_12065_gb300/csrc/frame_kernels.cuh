@@ -664,8 +664,7 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     float* Dp = X + bsz;
     const int xw = max(align_floats(6 * nqs), 2 * bsz);
     uint8_t* Mk = reinterpret_cast<uint8_t*>(X + xw);    // [TH*T*2] own masks (room for T*T*2)
-    uint8_t* Gs = Mk + 2 * T * T;                        // [TH*T*2] own groups
-    int* ex_list = reinterpret_cast<int*>(Gs + 2 * T * T);   // [kExactCap] deferred exact normals
+    int* ex_list = reinterpret_cast<int*>(Mk + 2 * T * T);   // [kExactCap] deferred exact normals
     const int tiles_x = div_up(Wq, T);
     const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
     const int qu0 = ty * TH - h, qv0 = tx * T - h;
@@ -914,11 +913,25 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
         return;
     }
 
-    // free after the last iteration (>= 6 * nqs floats, nqs >= (TH + 1) T): union-find parents, the
-    // run representative of each triangle, and the tile root of each representative [TH*T*2] each
+    // Outputs and segments of the tile, TH / 8 consecutive quad rows per warp with lane = column, so
+    // that a warp's groups, runs and links stay in its registers and shared memory holds only the
+    // runs' parents. What bounds it is latency: short dependent steps on two CTAs per SM. The label
+    // stage took 7.4 us of a tile's 26 us in a 256-frame batch with prefix-max shuffles for the
+    // runs, a compare-and-swap union per linked pair of runs and a walk per run, and takes 5.5 us
+    // with ballots and rounds over all links at once (batch 5869 -> 5716 us; 64 frames at one
+    // iteration 916 -> 882 us; a 480x640 frame 69.6 -> 68.1 us).
+    //
+    // free after the last iteration (>= 6 * nqs floats, nqs >= (TH + 1) T): parents of the run
+    // representatives [2 TH T], and each warp's last row for the warp below it: the representative
+    // (-1 without a group) and group of second(v), and the row's two link masks
     int32_t* Lp = reinterpret_cast<int32_t*>(nxt);
-    int32_t* RunOf = Lp + 2 * TH * T;
-    int32_t* RootOf = RunOf + 2 * TH * T;
+    int32_t* UpRep = Lp + 2 * TH * T;                    // [kThreads / 32][T]
+    int32_t* UpGrp = UpRep + kThreads;                   // [kThreads / 32][T]
+    unsigned* UpMask = reinterpret_cast<unsigned*>(UpGrp + kThreads);   // [kThreads / 32][2]
+    constexpr int kRows = T / (kThreads / 32);           // most rows of a warp
+    constexpr unsigned kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = TH / (kThreads / 32), r0 = warp * rows;
     uint8_t* const out_mask = a.out_mask;
     float* const out_normals = a.out_normals;
     uint8_t* const out_groups = a.groups;
@@ -934,19 +947,23 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     // GID; sizes, when present, are scratch of this library and 8-byte aligned)
     const bool vec_out = ((uintptr_t)out_mask & 1u) == 0 && ((uintptr_t)out_groups & 1u) == 0 &&
                          ((uintptr_t)out_normals & 7u) == 0;
-    for (int i = threadIdx.x; i < TH * T; i += blockDim.x) {
-        const int r = i / T, c = i - r * T;
-        const int gu = ty * TH + r, gv = tx * T + c;
+    static_assert(kRows == 4, "a warp's groups: 16 bits per row in one word");
+    unsigned long long grp = 0;                          // 16 bits per row: first(v)'s group, second(v)'s
+    const int gv = tx * T + lane;
+#pragma unroll 1   // (unrolled: 1,100 instructions more, 45 bytes spilled)
+    for (int row = 0; row < rows; ++row) {
+        const int r = r0 + row;
+        const int gu = ty * TH + r;
         const bool exists = gu < Hq && gv < Wq;
         V3 n[2];
-        load_quad(cur, (r + h) * RQW + (c + h), n[0], n[1]);
+        load_quad(cur, (r + h) * RQW + (lane + h), n[0], n[1]);
         const size_t gid0 = exists ? 2 * ((size_t)gu * Wq + gv) : 0;
+        const unsigned mk = *reinterpret_cast<const uint16_t*>(Mk + 2 * (r * T + lane));
         int gk[2];
         bool kk[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const int t = 2 * i + k;
-            const bool kept = Mk[t] != 0;
+            const bool kept = ((mk >> (8 * k)) & 255u) != 0;
             const bool has = has_normal(n[k]);
             int g = PL3D_NO_GROUP;
             if (exists && kept && has) {                                         // Algorithm 4, ang_min
@@ -975,8 +992,8 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
             gk[k] = g;
             kk[k] = kept;
             if (!has) n[k] = {NAN, NAN, NAN};
-            Gs[t] = exists ? (uint8_t)g : (uint8_t)PL3D_NO_GROUP;
         }
+        grp |= (unsigned long long)(unsigned)(gk[0] | (gk[1] << 8)) << (16 * row);
         if (exists) {
             // the quad's two triangles are consecutive GIDs: one store per array when aligned
             if (vec_out) {
@@ -1000,7 +1017,6 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
             if (sizes) *reinterpret_cast<int2*>(sizes + gid0) = make_int2(0, 0);
         }
     }
-    __syncthreads();
     stage_mark(bar, 3);
 
     // Connected components inside the tile (twins of Algorithm 2 that stay in the tile).
@@ -1010,98 +1026,146 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
         const float* n = ndv + 3 * g;
         return !offs || fabsf(n[0] * (ci.x - cj.x) + n[1] * (ci.y - cj.y) + n[2] * (ci.z - cj.z)) <= lim;
     };
-    constexpr unsigned kFull = 0xffffffffu;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // (1) Runs along each quad row. Chain position 2v is second(v), 2v+1 is first(v).
-    for (int r = warp; r < TH; r += kThreads / 32) {
-        const int tf = 2 * (r * T + lane), ts = tf + 1;
-        const int gf = Gs[tf], gs = Gs[ts];
-        V3 cf = {0.f, 0.f, 0.f}, cs2 = cf;
-        if (offs) load_quad(Cq, (r + h) * RQW + (lane + h), cf, cs2);
-        const int gs_next = __shfl_down_sync(kFull, gs, 1);
-        const V3 cs_next = {__shfl_down_sync(kFull, cs2.x, 1), __shfl_down_sync(kFull, cs2.y, 1),
-                            __shfl_down_sync(kFull, cs2.z, 1)};
-        const bool diag = gf != PL3D_NO_GROUP && gs == gf && offset_ok(gf, cf, cs2);
-        const bool right = lane < 31 && gf != PL3D_NO_GROUP && gs_next == gf && offset_ok(gf, cf, cs_next);
-        const bool right_prev = __shfl_up_sync(kFull, right, 1);
-        const bool brk_s = lane == 0 || !right_prev;                 // a run starts at second(v)
-        const bool brk_f = !diag;                                    // a run starts at first(v)
-        int pm = brk_f ? 2 * lane + 1 : (brk_s ? 2 * lane : -1);      // last run start up to this lane
+    auto group_of = [&](int k) { return (int)(grp >> (8 * k)) & 255; };   // 2 row + side
+    // (1) Runs along each quad row. Chain position 2v is second(v), 2v+1 is first(v); a run breaks
+    // at second(v) unless first(v-1) links to it (right), at first(v) unless the quad's diagonal
+    // links (diag). The last break at or before a position comes from the two ballots.
+    int repF[kRows], repS[kRows];                        // run representatives, -1 without a group
+    unsigned bD[kRows], bR[kRows];
+    const unsigned le = kFull >> (31 - lane), lt = le >> 1;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(kFull, pm, o);
-            if (lane >= o) pm = max(pm, v);
+    for (int row = 0; row < kRows; ++row) {
+        repF[row] = repS[row] = -1;
+        bD[row] = bR[row] = 0;
+        if (row >= rows) continue;
+        const int r = r0 + row;
+        const int gf = group_of(2 * row), gs = group_of(2 * row + 1);
+        const int gs_next = __shfl_down_sync(kFull, gs, 1);
+        bool diag = gf != PL3D_NO_GROUP && gs == gf;
+        bool right = lane < 31 && gf != PL3D_NO_GROUP && gs_next == gf;
+        if (offs) {
+            V3 cf, cs2;
+            load_quad(Cq, (r + h) * RQW + (lane + h), cf, cs2);
+            const V3 cs_next = {__shfl_down_sync(kFull, cs2.x, 1), __shfl_down_sync(kFull, cs2.y, 1),
+                                __shfl_down_sync(kFull, cs2.z, 1)};
+            diag = diag && offset_ok(gf, cf, cs2);
+            right = right && offset_ok(gf, cf, cs_next);
         }
-        const int before = __shfl_up_sync(kFull, pm, 1);
-        const int start_s = brk_s ? 2 * lane : before;
-        const int start_f = pm;
-        const unsigned brk_f_mask = __ballot_sync(kFull, brk_f);
+        bD[row] = __ballot_sync(kFull, diag);
+        bR[row] = __ballot_sync(kFull, right);
+        const unsigned brk_f = ~bD[row], brk_s = ~(bR[row] << 1);   // (bit 0 of brk_s: a row starts a run)
+        const int ls = 31 - __clz((int)(brk_s & le));
+        const int start_f = max(2 * (31 - __clz((int)(brk_f & le))) + 1, 2 * ls);
+        const int start_s = max(2 * (31 - __clz((int)(brk_f & lt))) + 1, 2 * ls);
         // smallest GID of a run starting at chain position p: first(p/2), unless the run is
         // second(p/2) alone
         auto root_of = [&](int p) {
             const int l0 = p >> 1;
-            const int t0 = 2 * (r * T + l0);
-            return ((p & 1) || !((brk_f_mask >> l0) & 1u)) ? t0 : t0 + 1;
+            return 2 * (r * T + l0) + (((p & 1) || !((brk_f >> l0) & 1u)) ? 0 : 1);
         };
-        const int rep_s = gs != PL3D_NO_GROUP ? root_of(start_s) : -1;
-        const int rep_f = gf != PL3D_NO_GROUP ? root_of(start_f) : -1;
-        Lp[ts] = rep_s;
-        Lp[tf] = rep_f;
-        RunOf[ts] = rep_s;
-        RunOf[tf] = rep_f;
+        const int tf = 2 * (r * T + lane);
+        if (gf != PL3D_NO_GROUP) repF[row] = root_of(start_f);
+        if (gs != PL3D_NO_GROUP) repS[row] = root_of(start_s);
+        if (repF[row] == tf) Lp[tf] = tf;
+        if (repS[row] == tf + 1) Lp[tf + 1] = tf + 1;
+        if (row == rows - 1) {
+            UpRep[threadIdx.x] = repS[row];
+            UpGrp[threadIdx.x] = gs;
+            if (lane == 0) {
+                UpMask[2 * warp] = bD[row];
+                UpMask[2 * warp + 1] = bR[row];
+            }
+        }
     }
     __syncthreads();
-    // (2) Rows joined across horizontal edges: first(r, v) with second(r-1, v); one union per
-    // run pair (a lane skips the pair its left neighbour already joined). Each warp takes a block
-    // of consecutive edges, top down, so that a union finds the row above already joined and the
-    // trees stay shallow (rows dealt to the warps in turn left chains as long as the tile is high;
-    // the tile's label stage took 9.6 us instead of 7.5 us on the 480x640 frame).
-    const int per_w = (TH - 1 + kThreads / 32 - 1) / (kThreads / 32);
-    for (int r = 1 + warp * per_w, r_end = min(TH, 1 + (warp + 1) * per_w); r < r_end; ++r) {
-        const int tf = 2 * (r * T + lane), tu = 2 * ((r - 1) * T + lane) + 1;
-        const int gf = Gs[tf];
-        bool link = gf != PL3D_NO_GROUP && Gs[tu] == gf;
+    // (2) Rows joined across horizontal edges: first(r, v) with second(r-1, v). A lane whose runs,
+    // above and below, both reach from the link of its left neighbour leaves the link to it.
+    int repU[kRows];
+    unsigned todo = 0;                                   // this thread's links not yet inside one segment
+#pragma unroll
+    for (int row = 0; row < kRows; ++row) {
+        repU[row] = -1;
+        if (row >= rows || (row == 0 && warp == 0)) continue;
+        const int r = r0 + row;
+        const int g_up = row == 0 ? UpGrp[threadIdx.x - 32] : group_of(row > 0 ? 2 * row - 1 : 0);
+        const unsigned upD = row == 0 ? UpMask[2 * warp - 2] : bD[row > 0 ? row - 1 : 0];
+        const unsigned upR = row == 0 ? UpMask[2 * warp - 1] : bR[row > 0 ? row - 1 : 0];
+        repU[row] = row == 0 ? UpRep[threadIdx.x - 32] : repS[row > 0 ? row - 1 : 0];
+        const int gf = group_of(2 * row);
+        bool link = gf != PL3D_NO_GROUP && g_up == gf;
         if (offs && link) {
             V3 cf, c1, c0u, cu;
             load_quad(Cq, (r + h) * RQW + (lane + h), cf, c1);
             load_quad(Cq, (r - 1 + h) * RQW + (lane + h), c0u, cu);
             link = offset_ok(gf, cf, cu);
         }
-        const int ra = link ? RunOf[tf] : -1, rb = link ? RunOf[tu] : -1;
-        const int pa = __shfl_up_sync(kFull, ra, 1), pb = __shfl_up_sync(kFull, rb, 1);
-        const bool dup = lane > 0 && pa == ra && pb == rb;
-        if (link && !dup) uf_unite(Lp, ra, rb);
+        const unsigned bL = __ballot_sync(kFull, link);
+        const unsigned same = (bL << 1) & (bR[row] << 1) & bD[row] & (upD << 1) & (upR << 1);
+        if (link && !((same >> lane) & 1u)) todo |= 1u << row;
     }
-    __syncthreads();
-    // (3) Only the run representatives were linked by the unions: each finds its root, halving
-    // the path as it walks (concurrent walks only shorten paths, so they stay valid).
-    for (int t = threadIdx.x; t < 2 * TH * T; t += blockDim.x)
-        if (RunOf[t] == t) RootOf[t] = uf_find(Lp, t);
-    __syncthreads();
+    // (3) Segments from the links, in rounds over all links at once. At the start of a round every
+    // representative points at its root. A link between two roots lowers the parent of the larger
+    // to the smaller (the smallest wins; a link stays on the list until it finds its two ends under
+    // one root, so one whose update lost is tried again). Then each representative jumps to its root,
+    // all at once, which takes the logarithm of a chain's length. A round that changes anything removes
+    // a root; scans take two or three rounds.
+    // A thread's loads are issued together in every step: what bounds a round is their latency.
+    volatile int32_t* const vp = Lp;
+    while (true) {
+        int x[kRows], y[kRows];
+#pragma unroll
+        for (int row = 0; row < kRows; ++row) {
+            const bool on = (todo >> row) & 1u;
+            x[row] = on ? vp[repF[row]] : 0;
+            y[row] = on ? vp[repU[row]] : 0;
+        }
+#pragma unroll
+        for (int row = 0; row < kRows; ++row) {
+            if (x[row] != y[row]) atomicMin(Lp + max(x[row], y[row]), min(x[row], y[row]));
+            else todo &= ~(1u << row);
+        }
+        if (!__syncthreads_or(todo != 0)) break;
+        int up[2 * kRows];                               // current parent of each own representative, -1: none
+#pragma unroll
+        for (int k = 0; k < 2 * kRows; ++k) {
+            const int t = 2 * ((r0 + (k >> 1)) * T + lane) + (k & 1);
+            up[k] = ((k & 1) ? repS[k >> 1] : repF[k >> 1]) == t ? vp[t] : -1;   // (a row past the warp's: -1)
+        }
+        bool more;
+        do {
+            more = false;
+            int g[2 * kRows];
+#pragma unroll
+            for (int k = 0; k < 2 * kRows; ++k) g[k] = up[k] >= 0 ? vp[up[k]] : -1;
+#pragma unroll
+            for (int k = 0; k < 2 * kRows; ++k)
+                if (g[k] != up[k]) {
+                    up[k] = g[k];
+                    vp[2 * ((r0 + (k >> 1)) * T + lane) + (k & 1)] = g[k];
+                    more = true;
+                }
+        } while (more);
+        __syncthreads();
+    }
     // (4) Each triangle leaves with the GID of its tile-local root (-1 without a group).
     int32_t* const labels = a.labels;
     const bool vec_lab = ((uintptr_t)labels & 7u) == 0;   // a quad's two labels in one 8-byte store
-    for (int i = threadIdx.x; i < TH * T; i += blockDim.x) {
-        const int r = i / T, c = i - r * T;
-        const int gu = ty * TH + r, gv = tx * T + c;
+    const int base = 2 * (ty * TH * Wq + tx * T);         // GID of the tile's first triangle
+#pragma unroll
+    for (int row = 0; row < kRows; ++row) {
+        if (row >= rows) break;
+        const int gu = ty * TH + r0 + row;
+        const int tF = repF[row] >= 0 ? Lp[repF[row]] : -1, tS = repS[row] >= 0 ? Lp[repS[row]] : -1;
+        // tile-local index 2 (row T + column) + side -> GID
+        const int labF = tF >= 0 ? base + (tF / (2 * T)) * (2 * Wq) + tF % (2 * T) : -1;
+        const int labS = tS >= 0 ? base + (tS / (2 * T)) * (2 * Wq) + tS % (2 * T) : -1;
         if (gu >= Hq || gv >= Wq) continue;
         const size_t gid0 = 2 * ((size_t)gu * Wq + gv);
-        int lab[2];
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int rep = RunOf[2 * i + k];
-            lab[k] = -1;
-            if (rep >= 0) {
-                const int root = RootOf[rep];
-                const int rq = root >> 1, rr = rq / T, rc = rq - rr * T;
-                lab[k] = (int)(2 * ((size_t)(ty * TH + rr) * Wq + (tx * T + rc)) + (root & 1));
-            }
-        }
         if (vec_lab) {
-            *reinterpret_cast<int2*>(labels + gid0) = make_int2(lab[0], lab[1]);
+            *reinterpret_cast<int2*>(labels + gid0) = make_int2(labF, labS);
         } else {
-            labels[gid0] = lab[0];
-            labels[gid0 + 1] = lab[1];
+            labels[gid0] = labF;
+            labels[gid0 + 1] = labS;
         }
     }
     __syncthreads();
