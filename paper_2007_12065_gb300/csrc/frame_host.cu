@@ -179,6 +179,72 @@ static int lap_tile_h(int iters, bool first, int halo, int requested) {
 
 static int bil_tile_h(const Tuning& t) { return t.bil_tile_h > 0 ? t.bil_tile_h : kTile; }
 
+// Time of a phase of `tiles` tiles: rounds of two CTAs per SM (`paired` each), the last one cheaper
+// when it leaves each SM one CTA; with one CTA per SM, rounds of `alone`.
+static double phase_cost(long long tiles, int sms, int per_sm, double paired, double alone) {
+    if (per_sm < 2) return (double)((tiles + sms - 1) / sms) * alone;
+    const long long full = tiles / (2LL * sms), rest = tiles % (2LL * sms);
+    return (double)full * paired + (rest == 0 ? 0.0 : rest <= sms ? alone : paired);
+}
+
+// Tile heights of a single frame whose tuning leaves them open. A phase lasts as long as its
+// rounds of tiles, and a tile's time is a fixed part plus a part per row, so low tiles win where 32
+// rows would leave SMs idle (a 120x160 frame has 20 such tiles for 304 CTAs: 49.7 us at 32 rows,
+// 36.1 us at 8-row bilateral tiles) or start one more round for a few tiles (720x1280: 920 tiles at
+// 32 rows, 1,200 at 24; 224 and 201 us), and tall ones where they save a round (its Laplacian at 48
+// rows: 224 and 206 us). The times below, in us, are a fit to such sweeps on a GB300 (2.07 GHz):
+// staging and geometry per staged row, iterations per row and iteration, groups and labels per
+// row; a tile alone on its SM takes 0.66 (bilateral) or 0.8
+// (Laplacian) of the time of each of two.
+Tuning frame_tuning(const Tuning& t, int H, int W, const pl3d_params* p, int dev) {
+    Tuning r = t;
+    int sms = 0;
+    if (H < 2 || W < 2 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+        return r;
+    constexpr double kBilAlone = 0.66, kLapAlone = 0.8;
+    const auto per_sm = [&](size_t smem) { return smem <= (size_t)kTwoCtaSmem && t.ctas_per_sm != 1 ? 2 : 1; };
+    if (t.bil_tile_h == 0) {
+        const int R = p->bil_iters > 0 ? p->bil_kernel / 2 : 1;
+        const int fuse = fused_iters(p->bil_iters, kBilMaxHalo / R, t.bil_fuse);
+        const int n = p->bil_iters < fuse ? p->bil_iters : fuse, h = n * R;
+        const double window = R == 1 ? 0.15 : R == 2 ? 0.36 : 0.7;
+        double best = 0.0;
+        for (int th = kBilMaxTileH; th >= kBilMinTileH; th -= 8) {
+            double paired = 6.7 + 0.216 * (th + 2 * h) * (kTile + 2 * h) / 38.0 + 0.16 * th;
+            for (int i = 1; i <= n; ++i)
+                paired += window * (th + 2 * (h - i * R)) * (kTile + 2 * (h - i * R)) / 34.0;
+            const long long tiles = (long long)div_up(H - 1, th) * div_up(W - 1, kTile);
+            const double c = phase_cost(tiles, sms, per_sm(bil_smem(h, th)), paired, kBilAlone * paired);
+            if (r.bil_tile_h == 0 || c < best) {
+                best = c;
+                r.bil_tile_h = th;
+            }
+        }
+    }
+    if (t.lap_tile_h == 0) {
+        const int R = p->lap_iters > 0 ? p->lap_kernel / 2 : 1;
+        const int fuse = fused_iters(p->lap_iters, kLapMaxHalo / R, t.lap_fuse);
+        const int n = p->lap_iters < fuse ? p->lap_iters : fuse, h = n * R;
+        // (a single-iteration pass keeps its own rule, lap_tile_h)
+        const double window = R == 1 ? 0.06 : R == 2 ? 0.14 : 0.28;
+        double best = 0.0;
+        for (int th = kLapMinTileH; n > 1 && th <= kLapMaxTileH; th += 8) {
+            const size_t smem = lap_smem_for(lap_box_floats(h, th), 1, 2);
+            if (th > kTile && smem > (size_t)kTwoCtaSmem) break;
+            double paired = 3.0;
+            for (int i = 1; i <= n; ++i)
+                paired += window * (th + 2 * (h - i * R)) * (kTile + 2 * (h - i * R)) / 36.0;
+            const long long tiles = (long long)div_up(H, th) * div_up(W, kTile);
+            const double c = phase_cost(tiles, sms, per_sm(smem), paired, kLapAlone * paired);
+            if (r.lap_tile_h == 0 || c < best) {
+                best = c;
+                r.lap_tile_h = th;
+            }
+        }
+    }
+    return r;
+}
+
 size_t border_counters(int H, int W, const Tuning& t) {
     if (H < 2 || W < 2) return 0;
     return 2 * (size_t)div_up(H - 1, bil_tile_h(t)) * (size_t)div_up(W - 1, kTile);

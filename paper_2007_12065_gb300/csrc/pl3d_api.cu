@@ -72,11 +72,12 @@ int run(pl3d_ctx* ctx, const float* points, int H, int W, const pl3d_params* p, 
         cudaStream_t s, int32_t* out_labels_copy = nullptr, cudaEvent_t normals_ready = nullptr) {
     const size_t npts = (size_t)H * W;
     const size_t ntri = 2 * (size_t)(H - 1) * (W - 1);
+    const Tuning t = frame_tuning(ctx->tuning, H, W, p, ctx->device);
     int rc;
     if ((rc = grow(&ctx->disp, &ctx->cap_points, npts, 6, s)) != PL3D_OK) return rc;
     if ((rc = grow_tri(ctx, ntri, s)) != PL3D_OK) return rc;
-    if ((rc = grow_border(ctx, border_counters(H, W, ctx->tuning), s)) != PL3D_OK) return rc;
-    if (bilateral_passes(p, ctx->tuning) > 1 && (rc = grow(&ctx->carry, &ctx->cap_carry, ntri, 6, s)) != PL3D_OK) return rc;
+    if ((rc = grow_border(ctx, border_counters(H, W, t), s)) != PL3D_OK) return rc;
+    if (bilateral_passes(p, t) > 1 && (rc = grow(&ctx->carry, &ctx->cap_carry, ntri, 6, s)) != PL3D_OK) return rc;
 
     FrameScratch sc;
     sc.disp[0] = ctx->disp;
@@ -111,11 +112,11 @@ int run(pl3d_ctx* ctx, const float* points, int H, int W, const pl3d_params* p, 
     record_start(ctx, s, &e0, &e1);
     int n_launched = 0;
     rc = frame_launch(sc, points, H, W, &q, nd_host, K, out_mask, out_normals, out_labels, out_points, out_groups,
-                      ctx->tuning, s, seeded ? nullptr : out_labels_copy, normals_ready, &n_launched);
+                      t, s, seeded ? nullptr : out_labels_copy, normals_ready, &n_launched);
     record_stop(ctx, s, kSlotKernel, e0, e1);
     if (rc != PL3D_OK) return rc;
     if (seeded) {
-        rc = seeded_labels(sc, final_disp(sc, &q, ctx->tuning), points, H, W, p, nd_host, K,
+        rc = seeded_labels(sc, final_disp(sc, &q, t), points, H, W, p, nd_host, K,
                            out_groups ? out_groups : ctx->groups, out_labels, s);
         if (rc != PL3D_OK) return rc;
         ctx->launches += 1;

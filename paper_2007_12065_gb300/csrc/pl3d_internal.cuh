@@ -241,11 +241,16 @@ struct Tuning {
     int lap_fuse;                  // most Laplacian iterations per pass, 0 = as many as fit the halo
     int bil_fuse;                  // same for the bilateral
     int ctas_per_sm;               // 0 = as many as fit
-    int lap_tile_h;                // Laplacian tile height in points, 0 = 32 (64 for a single-iteration
-                                   // first pass); a height whose buffers would not fit two CTAs per SM
-                                   // falls back to 32
-    int bil_tile_h;                // bilateral tile height in quads, 0 = 32
+    int lap_tile_h;                // Laplacian tile height in points, 0 = by frame_tuning for a single
+                                   // frame, 32 in a batch (64 for a single-iteration first pass); a
+                                   // height whose buffers would not fit two CTAs per SM falls back to 32
+    int bil_tile_h;                // bilateral tile height in quads, 0 = by frame_tuning for a single
+                                   // frame, 32 in a batch
 };
+
+// The tuning a single frame runs under: t with the tile heights it leaves open (0) chosen for the
+// frame's size and the device's SM count.
+Tuning frame_tuning(const Tuning& t, int H, int W, const pl3d_params* p, int dev);
 
 // Tile-border counters a frame's bilateral tiles use under tuning t (FrameArgs::border).
 size_t border_counters(int H, int W, const Tuning& t);
