@@ -48,18 +48,6 @@ constexpr int kPieces = kSlot / 4;
 static_assert(kLap1Cols == 64 && kLap1Rows % kBlock == 0, "warp tasks: 64 columns, whole blocks of rows");
 static_assert(kSlotPts + 3 * kLap1Cols + 3 <= kSlot && kPieces <= 64, "slot layout");
 
-__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // One row of the window: the point left of the lane's pair, the pair (a, b), the point right of it.
 struct L1Row {
     LapPt l, a, b, r;
