@@ -94,7 +94,8 @@ __device__ __forceinline__ void stage_box(float* dst, const float* src, const CU
 
 // ------------------------------------------------------------------------------ Laplacian
 
-// A Jacobi iteration updates strips of kLapStrip vertically adjacent points per thread: the
+// A Jacobi iteration of a 5 x 5 or 7 x 7 window updates strips of kLapStrip vertically adjacent
+// points per thread (a 3 x 3 window walks, see lap_walk): the
 // strip shares the loads of its (kLapStrip + 2R) x (2R + 1) window, and two strip points closer
 // than the radius share one weight (w_ij = w_ji, opposite differences).
 constexpr int kLapStrip = 4;
@@ -235,6 +236,83 @@ __device__ __forceinline__ void lap_issue(const FrameArgs& a, const LapPhase& ph
     mbar_arrive_expect_tx(bar, (unsigned)(ph.box.rows * ph.box.cols * 4));
     tma_load_2d(V0, map, o.x0, o.u0, bar);
 }
+// One Jacobi iteration with a 3 x 3 window over the region [lo, RH - lo) x [lo, RW - lo) of the staged
+// tile: from `cur` (displacements; unused when WITH_D = false) into `nxt`. Each thread walks down
+// one column of a segment of rows with a three-row window in registers: a row costs the loads of
+// three points, and its S edge is the next row's N edge. What bounds the pass is instruction issue
+// and the barrier after each iteration; the segments are cut so that every thread gets the same
+// number of rows (7, 6, 6, 5, 4 in five iterations of a 32 x 32 tile), where strips of four rows took
+// two rounds of the CTA for four of the five: 256 mixed frames 5723 -> 5656 us, 720x1280 181.6 ->
+// 179.8 us.
+// Every point takes its window in row-major order, so its sum does not depend on where the segments
+// fall (fused or split passes give the same bits).
+template <bool WITH_D>
+__device__ __forceinline__ void lap_walk(int H, int W, float lambda, int cols, const LapOrigin& og, int RH, int RW,
+                                         int lo, const float* V0, const float* cur, float* nxt) {
+    const int cw = RW - 2 * lo, nr = RH - 2 * lo;
+    const int segs = kThreads / cw;                      // (cw <= 48)
+    const int n = (nr + segs - 1) / segs;
+    const int seg = (int)threadIdx.x / cw;
+    const int c = lo + (int)threadIdx.x - seg * cw;
+    int r = lo + seg * n;
+    const int end = min(r + n, RH - lo);
+    if (seg >= segs || r >= end) return;
+    int o = r * cols + og.dlt + 3 * c;
+    const int gv = og.c0 + c;
+    const bool colpin = gv < 1 || gv >= W - 1;
+    struct Row {
+        LapPt l, c, r;
+    };
+    auto load = [&](Row& w, int at) {
+        w.l = lap_load<WITH_D>(V0, cur, at - 3);
+        w.c = lap_load<WITH_D>(V0, cur, at);
+        w.r = lap_load<WITH_D>(V0, cur, at + 3);
+    };
+    Row A, B, C;
+    load(A, o - cols);
+    load(B, o);
+    float ex, ey, ez;                                    // the edge from the point above to this one
+    lap_diff<WITH_D>(A.c, B.c, ex, ey, ez);
+    float w = lap_weight(ex, ey, ez);
+    auto step = [&](const Row& u, const Row& m, Row& d) {
+        load(d, o + cols);
+        LapAcc S;
+        S.c = m.c;
+        S.sx = S.sy = S.sz = S.ws = 0.f;
+        lap_add<WITH_D>(S, u.l);
+        S.sx = fmaf(-w, ex, S.sx);                       // fma(-w, e) = fma(w, -e)
+        S.sy = fmaf(-w, ey, S.sy);
+        S.sz = fmaf(-w, ez, S.sz);
+        S.ws = __fadd_rn(S.ws, w);
+        lap_add<WITH_D>(S, u.r);
+        lap_add<WITH_D>(S, m.l);
+        lap_add<WITH_D>(S, m.r);
+        lap_add<WITH_D>(S, d.l);
+        lap_diff<WITH_D>(m.c, d.c, ex, ey, ez);
+        w = lap_weight(ex, ey, ez);
+        lap_accumulate(S.sx, S.sy, S.sz, S.ws, w, ex, ey, ez);
+        lap_add<WITH_D>(S, d.r);
+        // Eq. 1 on the displacement; the pinned border ring, invalid points and points without a
+        // usable neighbour keep their displacement
+        const int gu = og.u0 + r;
+        const bool keep = colpin || gu < 1 || gu >= H - 1 || m.c.x == kInvalidCoord || !(S.ws > 0.f);
+        const float s = lap_scale(keep, lambda, S.ws);
+        nxt[o] = fmaf(s, S.sx, m.c.dx);
+        nxt[o + 1] = fmaf(s, S.sy, m.c.dy);
+        nxt[o + 2] = fmaf(s, S.sz, m.c.dz);
+        o += cols;
+        ++r;
+    };
+    while (true) {
+        step(A, B, C);
+        if (r == end) break;
+        step(B, C, A);
+        if (r == end) break;
+        step(C, A, B);
+        if (r == end) break;
+    }
+}
+
 // One Jacobi iteration (Eq. 1-2) over the region [lo, RH - lo) x [lo, RW - lo) of the staged
 // tile: from `cur` (displacements; unused when WITH_D = false) into `nxt`. A strip that runs
 // past the region's last row computes its extra points from the box's spare rows and discards
@@ -378,8 +456,13 @@ __device__ void lap_tile(const LapJob& j, float* V0, float* Da, float* Db, bool 
     float* cur = Da;
     float* nxt = Db;
     for (int t = 1; t <= j.iters; ++t) {
-        if (first && t == 1) lap_iteration<R, false>(H, W, j.lambda, b.cols, og, RH, RW, R, V0, cur, nxt);
-        else lap_iteration<R, true>(H, W, j.lambda, b.cols, og, RH, RW, t * R, V0, cur, nxt);
+        if constexpr (R == 1) {
+            if (first && t == 1) lap_walk<false>(H, W, j.lambda, b.cols, og, RH, RW, 1, V0, cur, nxt);
+            else lap_walk<true>(H, W, j.lambda, b.cols, og, RH, RW, t, V0, cur, nxt);
+        } else {
+            if (first && t == 1) lap_iteration<R, false>(H, W, j.lambda, b.cols, og, RH, RW, R, V0, cur, nxt);
+            else lap_iteration<R, true>(H, W, j.lambda, b.cols, og, RH, RW, t * R, V0, cur, nxt);
+        }
         __syncthreads();
         float* tmp = cur;
         cur = nxt;
