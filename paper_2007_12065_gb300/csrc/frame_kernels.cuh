@@ -1369,8 +1369,8 @@ __device__ __forceinline__ void merge_unite(int32_t* labels, bool link, int ra, 
 // between launches. Counter 2t is tile t's top border, 2t + 1 its left border. Warp k of the CTA
 // takes side k (top, left, bottom, right), its lanes along the border (merge_pair's items); the
 // other warps go on. Each item's groups and labels are loaded together; the unions halve the
-// paths they walk, which keeps the trees shallow for the flatten phase (walking both paths side by
-// side without halving measured 6 us slower per 480x640 frame, most of it in the flatten).
+// paths they walk, which keeps the trees shallow for the flatten phase (without halving: 6 us slower per
+// 480x640 frame, most of it in the flatten).
 __device__ __forceinline__ void join_tile_borders(const FrameArgs& a, int tile) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp >= 4) return;

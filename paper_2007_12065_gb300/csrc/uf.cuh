@@ -1,11 +1,10 @@
-// uf.cuh -- lock-free union-find over an int32 parent array (shared or global memory).
+// uf.cuh -- lock-free union-find over an int32 parent array in global memory.
 //
 // Every parent pointer points to a smaller-or-equal index, and a root is only linked below a
 // smaller root, with a compare-and-swap on the larger root. So each component ends with its
 // smallest index as root, whatever order the unions run in, and the result is deterministic.
-// Finding halves the path as it walks: each visited node is pointed at its grandparent, an
-// ancestor, so concurrent walks and links stay valid. Walks that run after all unions have
-// finished use the read-only form.
+// Walks halve the path: each visited node is pointed at its grandparent, an ancestor, so
+// concurrent walks and links stay valid.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -13,43 +12,27 @@
 
 namespace pl3d {
 
-__device__ __forceinline__ int uf_find(int32_t* L, int x) {
-    volatile int32_t* vl = L;
-    while (true) {
-        const int p = vl[x];
-        if (p == x) return x;
-        const int gp = vl[p];
-        if (gp == p) return p;
-        vl[x] = gp;
-        x = gp;
-    }
-}
-
+// What bounds a union is the latency of L2, several hundred cycles per step, so both paths are walked
+// together: one trip per step instead of two (and one trip and the swap for two roots). Against a walk per
+// end: 256 frames' merge phase 227 -> 162 us, a 240x320 frame 39.7 -> 38.9 us, 480x640 68.0 -> 66.8 us.
 __device__ __forceinline__ void uf_unite(int32_t* L, int a, int b) {
-    while (true) {
-        a = uf_find(L, a);
-        b = uf_find(L, b);
-        if (a == b) return;
-        if (a > b) {
-            const int t = a;
-            a = b;
-            b = t;
+    volatile int32_t* vl = L;
+    while (a != b) {
+        const int pa = vl[a], pb = vl[b];
+        if (pa == a && pb == b) {
+            const int hi = max(a, b), lo = min(a, b);
+            const int old = atomicCAS(L + hi, hi, lo);
+            if (old == hi) return;
+            a = old;   // hi stopped being a root meanwhile; continue from its new parent
+            b = lo;
+            continue;
         }
-        const int old = atomicCAS(L + b, b, a);
-        if (old == b) return;
-        b = old;   // b stopped being a root meanwhile; continue from its new parent
+        const int ga = vl[pa], gb = vl[pb];
+        if (ga != pa) vl[a] = ga;
+        if (gb != pb) vl[b] = gb;
+        a = ga;
+        b = gb;
     }
-}
-
-// Root of x when no union runs concurrently (reads only).
-__device__ __forceinline__ int uf_root(const int32_t* L, int x) {
-    const volatile int32_t* vl = L;
-    int p = vl[x];
-    while (p != x) {
-        x = p;
-        p = vl[x];
-    }
-    return x;
 }
 
 }  // namespace pl3d
