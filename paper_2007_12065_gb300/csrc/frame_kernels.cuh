@@ -700,9 +700,10 @@ __device__ __forceinline__ void quad_neighbour(QuadAcc& A, f2 a2, f2 cx, f2 cy, 
 // segments (Algorithm 5); with JOIN (the single-frame kernel) also the joins across the tile's
 // borders with finished neighbours.
 // Shared-memory header of the persistent kernels (128 bytes before the tiles' buffers): the staging
-// mbarriers from byte 0, the bilateral tile's deferred-normal count at byte 64, and for the stage
+// mbarriers from byte 0, the bilateral tile's deferred-normal count at byte 64, the grid barrier's
+// generation at byte 68, and for the stage
 // timing the last stamp at byte 72 and the stage totals' address (or nullptr) at byte 80.
-constexpr int kHdrExact = 64, kHdrStamp = 72, kHdrStages = 80;
+constexpr int kHdrExact = 64, kHdrGen = 68, kHdrStamp = 72, kHdrStages = 80;
 
 // The borders of a finished tile's segments with its neighbours' (defined with the merge phase).
 __device__ __forceinline__ void join_tile_borders(const FrameArgs& a, int tile);
@@ -1564,6 +1565,8 @@ __global__ void __launch_bounds__(kThreads, 2) frame_kernel(const __grid_constan
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);   // [kLapMaxStages]: one per staging slot
     float* smem = reinterpret_cast<float*>(smem_raw + 128);
+    unsigned* gen = reinterpret_cast<unsigned*>(smem_raw + frame::kHdrGen);
+    grid_barrier_begin(a.barrier, gen);
     if (threadIdx.x == 0)
         for (int i = 0; i < kLapMaxStages; ++i) mbar_init(bar + i, 1);
     frame::set_stage_timing(bar, a.phase_ns ? a.phase_ns + kStageSlot : nullptr);
@@ -1602,26 +1605,26 @@ __global__ void __launch_bounds__(kThreads, 2) frame_kernel(const __grid_constan
                 if (map) par ^= 1u << s;
                 s = s + 1 == ns ? 0 : s + 1;
             }
-            grid_barrier(a.barrier, a.error);
+            grid_barrier(a.barrier, a.error, gen);
         }
         frame::phase_mark(a, 0, t_prev);
         const int tiles_bil = div_up(a.H - 1, a.bil_th) * div_up(a.W - 1, kTile);
         unsigned par0 = par & 1u;   // the bilateral stages through slot 0
         for (int c = 0; c < a.n_bil; ++c) {
             for (int t = blockIdx.x; t < tiles_bil; t += gridDim.x) frame::bil_tile<RB, true>(a, a.bil[c], t, smem, bar, par0);
-            if (a.part == 0 || c + 1 < a.n_bil) grid_barrier(a.barrier, a.error);
+            if (a.part == 0 || c + 1 < a.n_bil) grid_barrier(a.barrier, a.error, gen);
         }
         frame::phase_mark(a, 1, t_prev);
     }
     if (a.part == 1) return;
     if (!a.border) {   // else the bilateral tiles joined their borders
         frame::merge_phase(a);
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, gen);
     }
     frame::phase_mark(a, 2, t_prev);
     frame::flatten_phase(a);
     if (a.min_triangles > 0) {
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, gen);
         frame::filter_phase(a);
     }
     frame::phase_mark(a, 3, t_prev);
@@ -1662,6 +1665,8 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);   // [kLapMaxStages]: one per staging slot
     float* smem = reinterpret_cast<float*>(smem_raw + 128);
+    unsigned* gen = reinterpret_cast<unsigned*>(smem_raw + frame::kHdrGen);
+    grid_barrier_begin(b.barrier, gen);
     if (threadIdx.x == 0)
         for (int i = 0; i < kLapMaxStages; ++i) mbar_init(bar + i, 1);
     frame::set_stage_timing(bar, b.hdr->timing ? b.phase_ns + kStageSlot : nullptr);
@@ -1738,7 +1743,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
             if (tma) par ^= 1u << s;
             s = s + 1 == ns ? 0 : s + 1;
         }
-        grid_barrier(b.barrier, b.error);
+        grid_barrier(b.barrier, b.error, gen);
     }
     mark(0);
     unsigned par0 = par & 1u;   // the bilateral stages through slot 0
@@ -1760,7 +1765,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
             }
             frame::bil_tile<RB, false>(a, a.bil[c], t - __ldg(pre + f), smem, bar, par0);
         }
-        grid_barrier(b.barrier, b.error);
+        grid_barrier(b.barrier, b.error, gen);
     }
     mark(1);
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1783,7 +1788,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
             frame::merge_unite(labels, link, ra, rb, f);
         }
     }
-    grid_barrier(b.barrier, b.error);
+    grid_barrier(b.barrier, b.error, gen);
     mark(2);
     {
         // every grouped triangle takes its root, block by block. Frame f's blocks start at
@@ -1800,7 +1805,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
         }
     }
     if (any_filter) {
-        grid_barrier(b.barrier, b.error);
+        grid_barrier(b.barrier, b.error, gen);
         // Algorithm 5 keeps a segment only when it has more than tri_min triangles
         const long long total = __ldg(b.tris + n);
         int f = 0;

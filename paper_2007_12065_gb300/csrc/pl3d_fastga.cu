@@ -494,6 +494,8 @@ constexpr int kGaBatch = 2;   // normals a thread loads before it locates them
 // barrier (every share cleared) it adds its histogram to the output.
 __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_constant__ GaArgs a) {
     extern __shared__ int hist[];   // [cells]
+    __shared__ unsigned gen;
+    grid_barrier_begin(a.barrier, &gen);
     for (int i = threadIdx.x; i < a.cells; i += blockDim.x) hist[i] = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.cells;
          i += (long long)gridDim.x * blockDim.x)
@@ -536,7 +538,7 @@ __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_cons
             if (a.out_cell && in_range[k]) a.out_cell[idx[k]] = cell;
         }
     }
-    grid_barrier(a.barrier, a.error);   // every CTA's share of the output cleared (and this CTA's hist final)
+    grid_barrier(a.barrier, a.error, &gen);   // every CTA's share of the output cleared (and this CTA's hist final)
     for (int i = threadIdx.x; i < a.cells; i += blockDim.x)
         if (hist[i]) atomicAdd(a.counts + i, hist[i]);
 }

@@ -162,6 +162,8 @@ __device__ __forceinline__ Flags gid_flags(const MeshArgs& a, long long g, long 
 __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant__ MeshArgs a) {
     __shared__ int sh_scan[kWarps + 1];
     __shared__ int sh_sum[2 * kWarps];
+    __shared__ unsigned sh_gen;
+    grid_barrier_begin(a.barrier, &sh_gen);
     // dynamic: digit counts [kMaxBins], digit bases [kMaxBins], per-warp digit counts
     // [kWarps][kMaxBins] (16-bit: at most kChunk / kWarps entries per warp)
     extern __shared__ int mesh_smem[];
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
             cR[c] = tr;
         }
     }
-    grid_barrier(a.barrier, a.error);
+    grid_barrier(a.barrier, a.error, &sh_gen);
 
     // every CTA sums the chunk counts it needs itself (no separate scan phase): the totals, and
     // below the counts of the chunks before each of its own
@@ -321,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nz; i += (long long)gridDim.x * blockDim.x)
             a.seg_chunk[i] = 0;
     }
-    grid_barrier(a.barrier, a.error);
+    grid_barrier(a.barrier, a.error, &sh_gen);
 
     // D: HE (Algorithm 2) and the sort keys
     {
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
         if (a.labels && blockIdx.x == 0 && threadIdx.x == 0) a.seg_offsets[0] = 0;
         return;
     }
-    grid_barrier(a.barrier, a.error);
+    grid_barrier(a.barrier, a.error, &sh_gen);
 
     if (one) {
         const int ln = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -444,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
                 if (ln == 0) a.seg_cnt[k] = carry;
             }
         }
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, &sh_gen);
         // P: stable scatter into the segment lists; the CSR offsets are the segment starts
         int* const sh_start = mesh_smem;                                                  // [kMaxOnePass]
         uint16_t* const wc = reinterpret_cast<uint16_t*>(mesh_smem + kMaxOnePass);       // [kWarps][kMaxOnePass]
@@ -542,7 +544,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
             for (int d = threadIdx.x; d < bins; d += kThreads) a.hist[(long long)d * Ct + c] = sh_bins[d];
             __syncthreads();
         }
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, &sh_gen);
         // R2: per digit, exclusive offsets over the chunks, and the digit's total
         for (int d = blockIdx.x; d < bins; d += gridDim.x) {
             int32_t* h = a.hist + (long long)d * Ct;
@@ -557,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
             }
             if (threadIdx.x == 0) a.bin_tot[d] = (int)carry;
         }
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, &sh_gen);
         // R3: stable scatter
         {
             int tot;
@@ -617,7 +619,7 @@ __global__ void __launch_bounds__(kThreads, 4) mesh_kernel(const __grid_constant
             }
             __syncthreads();
         }
-        grid_barrier(a.barrier, a.error);
+        grid_barrier(a.barrier, a.error, &sh_gen);
     }
 
     // G: CSR of the segments (their boundary half-edges came with HE in D)

@@ -23,7 +23,9 @@ constexpr int kKindMbarrier = 2;
 __global__ void wait_selftest_kernel(unsigned* bar, int* err, int kind, unsigned long long limit_ns) {
     if (kind == kKindBarrier) {
         if (blockIdx.x == gridDim.x - 1) return;   // leaves without arriving at the barrier
-        grid_barrier(bar, err, limit_ns);
+        __shared__ unsigned gen;
+        grid_barrier_begin(bar, &gen);
+        grid_barrier(bar, err, &gen, limit_ns);
     } else if (kind == kKindMbarrier && blockIdx.x == 0) {
         __shared__ __align__(8) uint64_t mb;
         if (threadIdx.x == 0) mbar_init(&mb, 1);
