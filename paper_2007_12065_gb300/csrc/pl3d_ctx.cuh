@@ -34,10 +34,13 @@ struct BatchGraph {
     cudaGraphExec_t exec;
 };
 
-// barrier [2], error word, pad; phase totals [4]; lap1 timing stamps [3]; bilateral stage totals
+// barrier count, unused, error word, barrier count; phase totals [4]; lap1 timing stamps [3]; bilateral
+// stage totals
 // [5] (u64); lap1 task counter [2]
-constexpr size_t kCtlBytes =
+constexpr size_t kCtlUsed =
     4 * sizeof(unsigned) + (kStageSlot + kBilStages) * sizeof(unsigned long long) + 2 * sizeof(unsigned);
+static_assert(kCtlUsed <= 32 * sizeof(unsigned), "word 32 (the barrier's generation, sync.cuh) is free");
+constexpr size_t kCtlBytes = 64 * sizeof(unsigned);
 
 }  // namespace ctxutil
 }  // namespace pl3d

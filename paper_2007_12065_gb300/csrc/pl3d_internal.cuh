@@ -10,7 +10,7 @@
 //   groups           u8   [2Q]                (scratch or the caller's buffer)
 //   labels           i32  [2Q]                (caller's buffer; doubles as the union-find parents)
 //   segment sizes    i32  [2Q]                (scratch, only when tri_min > 0)
-//   barrier, error   u32 [2], i32             (scratch: grid barrier state, device error word)
+//   control words    u32                      (scratch: grid barrier state (sync.cuh), device error word)
 #pragma once
 
 #include <cuda.h>
@@ -131,7 +131,7 @@ struct FrameArgs {
     float max_offset;              // <= 0 when disabled
     float max_offset_scaled;       // max_offset * c_scale
     int min_triangles;
-    unsigned* barrier;             // [2] grid barrier state
+    unsigned* barrier;             // grid barrier state (sync.cuh)
     int* error;                    // device error word (sync.cuh bits)
     unsigned* border;              // [2 x bilateral tiles], even between launches: counters of the tile
                                    // borders that the bilateral tiles join themselves; nullptr: the
@@ -225,7 +225,7 @@ struct FrameScratch {
     float* carry[2];               // >= 6 Q floats each when the bilateral needs several passes
     uint8_t* groups;               // >= 2 Q
     int32_t* sizes;                // >= 2 Q
-    unsigned* barrier;             // [2], zero before the first use
+    unsigned* barrier;             // control words (sync.cuh), zero before the first use
     int* error;                    // [1]
     unsigned long long* phase_ns;  // [4] or nullptr
     unsigned* lap1_sched;          // [2], zero at rest: the single-iteration Laplacian's task counter
@@ -324,7 +324,7 @@ int frame_launch(const FrameScratch& sc, const float* points, int H, int W, cons
                  uint8_t* out_groups, const Tuning& t, cudaStream_t s, int32_t* out_labels_copy = nullptr,
                  cudaEvent_t normals_ready = nullptr, int* launches = nullptr);
 
-// Device address of the allocation-free entry point's control words (barrier [2], error word,
+// Device address of the allocation-free entry point's control words (barrier, error word,
 // pad) on the current device (pl3d_static.cu).
 int static_control_words(unsigned** ctl);
 

@@ -40,7 +40,7 @@ constexpr size_t kMaxTri = 2 * kMaxPoints;                       // 2(H-1)(W-1) 
 constexpr size_t kDispBytes = 6 * kMaxPoints * sizeof(float);    // displacement ping-pong, AoS
 constexpr size_t kGroupBytes = (kMaxTri + 255) / 256 * 256;
 constexpr size_t kSizeBytes = kMaxTri * sizeof(int32_t);
-constexpr size_t kCtlBytes = 256;                                // barrier [2], error word, pad,
+constexpr size_t kCtlBytes = 256;                                // barrier, error word,
                                                                  // lap1 task counter [2]
 constexpr size_t kScratchBytes = kDispBytes + kGroupBytes + kSizeBytes + kCtlBytes;
 
@@ -89,7 +89,7 @@ constexpr size_t kCtlOffset = kDispBytes + kGroupBytes + kSizeBytes;
 
 namespace pl3d {
 
-// Device address of the allocation-free path's control words (barrier [2], error word, pad) on
+// Device address of the allocation-free path's control words (barrier, error word) on
 // the current device, after the same once-per-device set-up as the entry point.
 int static_control_words(unsigned** ctl) {
     int dev = -1;

@@ -121,19 +121,26 @@ __device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Grid-wide barrier for a co-resident (cooperatively launched) grid. bar[0] counts arrivals,
-// bar[1] is the generation. Thread 0 of each CTA arrives with an acquire-release add, which
+// Grid-wide barrier for a co-resident (cooperatively launched) grid. The control words hold two
+// counts of arrivals, used in turn, and the generation, on a line of its own (the waiting CTAs
+// poll it while others arrive). Thread 0 of each CTA arrives with an acquire-release add, which
 // publishes the writes its CTA made before the __syncthreads (cumulativity) and, for the last
-// arriver, acquires everyone else's; the last arriver resets the count and opens the barrier
-// with a release add on the generation, which the others wait for with acquire loads. Global
-// writes made before the barrier are visible to every thread of the grid after it.
+// arriver, acquires everyone else's; the last arriver opens the barrier with a release add on the
+// generation, which the others wait for with acquire loads, and then resets the count: nobody adds
+// to it again before the next barrier, on the other count, has passed, which orders the reset.
+// Global writes made before the barrier are visible to every thread of the grid after it.
 //
-// The generation cannot advance before this CTA arrives, so its value is fetched once, at the start
-// of the kernel (grid_barrier_begin: an asynchronous copy into `gen`, a word of shared memory), and
-// counted from there: read at each barrier it put a trip to L2 before every arrival (64x1024 frame 34.7
-// -> 33.5 us, 240x320 38.9 -> 37.3 us with two barriers, mesh of 480x640 38.4 -> 37.7 us with four).
+// What bounds it is three trips to L2 (the last arrival, the opening, the poll that sees it), 1.7 us
+// for 20 to 304 CTAs. The generation cannot advance before this CTA arrives, so its value is fetched
+// once, at the start of the kernel (grid_barrier_begin: an asynchronous copy into `gen`, a word of
+// shared memory), and counted from there: read at each barrier it put a fourth trip before every
+// arrival (64x1024 frame 34.7 -> 33.5 us with two barriers, mesh of 480x640 38.4 -> 37.7 us with four).
+// A reset before the opening, on one count, held the opening back by its own trip, and the polls ran into
+// the arrivals on one line (mesh 36.9 -> 36.1 us, 480x640 frame 66.1 -> 65.9 us).
+constexpr int kBarrierGen = 32;      // word of the generation; the counts are words 0 and 3
+
 __device__ __forceinline__ void grid_barrier_begin(const unsigned* bar, unsigned* gen) {
-    if (threadIdx.x == 0) cp_async4(reinterpret_cast<float*>(gen), reinterpret_cast<const float*>(bar + 1));
+    if (threadIdx.x == 0) cp_async4(reinterpret_cast<float*>(gen), reinterpret_cast<const float*>(bar + kBarrierGen));
 }
 
 // The two halves of a barrier, for work that fits between them (a CTA that has arrived must wait
@@ -142,10 +149,12 @@ __device__ __forceinline__ void grid_barrier_arrive(unsigned* bar, unsigned* gen
     __syncthreads();
     if (threadIdx.x == 0) {
         cp_async_wait_all();
-        *gen += 1u;
-        if (atom_add_acq_rel_gpu(bar, 1u) + 1u == gridDim.x * gridDim.y * gridDim.z) {
-            *reinterpret_cast<volatile unsigned*>(bar) = 0u;   // ordered before the release below
-            red_release_gpu_add(bar + 1, 1u);
+        const unsigned g = *gen;
+        *gen = g + 1u;
+        unsigned* const count = bar + 3u * (g & 1u);
+        if (atom_add_acq_rel_gpu(count, 1u) + 1u == gridDim.x * gridDim.y * gridDim.z) {
+            red_release_gpu_add(bar + kBarrierGen, 1u);
+            *reinterpret_cast<volatile unsigned*>(count) = 0u;
         }
     }
 }
@@ -155,7 +164,7 @@ __device__ __forceinline__ void grid_barrier_wait(unsigned* bar, int* err, const
     if (threadIdx.x == 0) {
         const unsigned g = *gen - 1u;   // the generation that the barrier's opening ends
         const uint64_t t0 = global_ns();
-        for (uint32_t i = 1; ld_acquire_gpu(bar + 1) == g; ++i) {
+        for (uint32_t i = 1; ld_acquire_gpu(bar + kBarrierGen) == g; ++i) {
             if ((i & 63u) == 0u && global_ns() - t0 > limit_ns) {
                 atomicOr(err, kErrBarrierTimeout);
                 break;
