@@ -327,7 +327,8 @@ int pl3d_extract_planes_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, 
  * changes a result bit: iterations split over more passes go through global memory as the same
  * FP32 values the fused form keeps in shared memory.
  *   lap_fuse     most Laplacian iterations fused into one tile pass (0 = as many as the tile's
- *                halo of 8 points allows); fewer means smaller halos but more passes.
+ *                halo of 8 points allows, or one per pass for a large batch with a 3 x 3 window);
+ *                fewer means smaller halos but more passes.
  *   bil_fuse     the same for the bilateral (halo of 6 quads).
  *                Either depth is raised where needed so that a filter takes at most 8 passes.
  *   ctas_per_sm  resident CTAs per SM of the persistent launch (0 = as many as fit, at most 2).
