@@ -52,7 +52,7 @@ size_t bil_smem(int halo, int th) {
     const int quads = align_floats(6 * (rh * rq + rq));
     const int boxes = 2 * align_floats(b.rows * b.cols);
     return 128 + 4 * (size_t)(2 * quads + (quads > boxes ? quads : boxes)) + 2 * (size_t)kTile * kTile +
-           4 * (size_t)kExactCap;
+           ((2 * (size_t)rh * rq + 15) & ~(size_t)15);
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda).

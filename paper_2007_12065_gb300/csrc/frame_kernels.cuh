@@ -756,7 +756,9 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     float* Dp = X + bsz;
     const int xw = max(align_floats(6 * nqs), 2 * bsz);
     uint8_t* Mk = reinterpret_cast<uint8_t*>(X + xw);    // [TH*T*2] own masks (room for T*T*2)
-    int* ex_list = reinterpret_cast<int*>(Mk + 2 * T * T);   // [kExactCap] deferred exact normals
+    uint16_t* ex_list = reinterpret_cast<uint16_t*>(Mk + 2 * T * T);   // [nq] deferred exact normals: quad | which
+    constexpr int kDefer0 = 1 << 12, kDefer1 = 1 << 13;
+    static_assert((T + 2 * kBilMaxHalo) * (T + 2 * kBilMaxHalo) <= kDefer0, "staged quads in 12 bits");
     const int tiles_x = div_up(Wq, T);
     const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
     const int qu0 = ty * TH - h, qv0 = tx * T - h;
@@ -819,9 +821,10 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     stage_mark(bar, 0);
 
     // Centroids and normals of every staged triangle; masks of the tile's own quads. A normal
-    // whose FP32 error bound fails is deferred: its quad goes on a short list that a second
-    // loop recomputes from exact pairs with every lane busy (inline, divergent, only when the
-    // list is full).
+    // whose FP32 error bound fails is deferred: its quad goes on a list (with room for every staged
+    // quad) that a second loop recomputes from exact pairs with every lane busy. On a LiDAR scan a fifth
+    // of the quads are; a list of 256 with a divergent path past it took 33.4 us for a 64x1024 frame
+    // and 868 us for 64 frames at one iteration, this one 33.1 and 863 us.
     auto exact_normals = [&](const SP& p1, const SP& p2, const SP& p3, const SP& p4, bool do0, bool do1, V3& n0,
                              V3& n1) {
         const PairEdge pd = pair_edge(p3, p1);
@@ -876,19 +879,11 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
             V3 cr0 = cross(er.e, ed.e), cr1 = cross(el.e, edn.e);
             const bool exact0 = valid0 && !fast_cross_ok(er, ed, cr0);
             const bool exact1 = valid1 && !fast_cross_ok(el, edn, cr1);
-            bool defer = false;
-            if (exact0 || exact1) {
-                const int slot = atomicAdd(n_exact, 1);
-                if (slot < kExactCap) {
-                    ex_list[slot] = q | (exact0 ? 1 << 29 : 0) | (exact1 ? 1 << 30 : 0);
-                    defer = true;
-                } else {
-                    exact_normals(p1, p2, p3, p4, exact0, exact1, cr0, cr1);
-                }
-            }
+            if (exact0 || exact1)
+                ex_list[atomicAdd(n_exact, 1)] = (uint16_t)(q | (exact0 ? kDefer0 : 0) | (exact1 ? kDefer1 : 0));
             // a deferred quad's records are written again by the second loop
-            nn[0] = unit_or_none(cr0, valid0 && !(defer && exact0));
-            nn[1] = unit_or_none(cr1, valid1 && !(defer && exact1));
+            nn[0] = unit_or_none(cr0, valid0 && !exact0);
+            nn[1] = unit_or_none(cr1, valid1 && !exact1);
         } else {
             const bool vk[2] = {valid0, valid1};
 #pragma unroll
@@ -916,11 +911,11 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     }
     __syncthreads();
     // the deferred normals (and their centroids), one quad per lane
-    const int n_ex = min(*n_exact, kExactCap);
+    const int n_ex = *n_exact;
     for (int i = threadIdx.x; i < n_ex; i += blockDim.x) {
         const int e = ex_list[i];
-        const int q = e & ((1 << 29) - 1);
-        const bool do0 = (e >> 29) & 1, do1 = (e >> 30) & 1;
+        const int q = e & (kDefer0 - 1);
+        const bool do0 = e & kDefer0, do1 = e & kDefer1;
         const int qr = q / RQW, qc = q - qr * RQW;
         const int o1 = qr * b.cols + dlt + 3 * qc;
         const SP p1 = load_sp(V0, Dp, o1), p2 = load_sp(V0, Dp, o1 + 3);

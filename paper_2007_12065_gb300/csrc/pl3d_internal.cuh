@@ -25,7 +25,6 @@ constexpr int kThreads = 256;    // threads per CTA
 constexpr int kTile = 32;        // tile edge: 32 x 32 points (Laplacian) or quads (bilateral)
 constexpr int kLapMaxHalo = 8;   // largest halo (fused iterations x radius) of one Laplacian pass
 constexpr int kBilMaxHalo = 6;   // same for the bilateral
-constexpr int kExactCap = 256;   // deferred exact-normal quads a bilateral tile lists (then inline)
 // Shared memory per CTA that still lets two CTAs share an SM (the bilateral pass at halo 3 needs
 // this much); a Laplacian pass stages as many boxes ahead as fit within it.
 constexpr int kTwoCtaSmem = 114048;
