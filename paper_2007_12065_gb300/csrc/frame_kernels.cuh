@@ -1412,8 +1412,8 @@ __device__ __forceinline__ void merge_phase(const FrameArgs& a) {
     }
 }
 
-// Flatten: every grouped triangle takes its root, in blocks of kFlatBlock consecutive labels per
-// warp, kFlatVec 16-byte loads per lane. A triangle's label is the root of its tile's segment, whose
+// Flatten: every grouped triangle takes its root, in blocks of 128 VEC consecutive labels per
+// warp, VEC 16-byte loads per lane. A triangle's label is the root of its tile's segment, whose
 // parent chain (one or two hops, measured) ends at the segment's root.
 //
 // What bounds it: most of a frame's chains end at a few roots (the floor, a wall), so thousands of
@@ -1423,24 +1423,29 @@ __device__ __forceinline__ void merge_phase(const FrameArgs& a) {
 // cached here is no older than the last union, and a word that another thread has meanwhile replaced
 // by its root was and is an ancestor, either way. The labels themselves are read once, past L1, 16
 // bytes per lane. With both, the phase took 0.38 ms and the batch 5.88 instead of 7.40 ms; a 480x640
-// frame 69.6 instead of 73.7 us.
-constexpr int kFlatVec = 2;
-constexpr int kFlatBlock = 32 * 4 * kFlatVec;
+// frame 69.6 instead of 73.7 us. After that a warp waits for one load after another, so a batch,
+// whose warps take dozens of blocks each, has kFlatVecBatch loads per lane in flight (417 us at 2, 278 us
+// at 4, 178 us at 8); a single frame has less than a block per warp, and 4 cost it 0.9 us.
+constexpr int kFlatVec = 2, kFlatVecBatch = 8;
+template <int VEC>
+constexpr int kFlatBlock = 32 * 4 * VEC;
 
 // Blocks of a frame of n labels; blocks start at 16-byte boundaries, up to 3 labels before the first.
-__device__ __forceinline__ long long flatten_blocks(long long n) { return (n + 3 + kFlatBlock - 1) / kFlatBlock; }
+template <int VEC>
+__device__ __forceinline__ long long flatten_blocks(long long n) { return (n + 3 + kFlatBlock<VEC> - 1) / kFlatBlock<VEC>; }
 
 // Block b of the labels L[0 .. n): roots into L and, when given, into `copy`; with `sizes` the
 // segment sizes are counted (an atomic per root and warp load, one per block when it has one root).
 // Called by whole warps.
+template <int VEC>
 __device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* sizes, int32_t* copy, long long b) {
     const int lane = threadIdx.x & 31;
     const int shift = (int)(((uintptr_t)L >> 2) & 3u);
-    const long long i0 = b * kFlatBlock - shift + 4 * lane;
-    int x[4 * kFlatVec], p[4 * kFlatVec];
-    bool whole[kFlatVec];
+    const long long i0 = b * kFlatBlock<VEC> - shift + 4 * lane;
+    int x[4 * VEC], p[4 * VEC];
+    bool whole[VEC];
 #pragma unroll
-    for (int v = 0; v < kFlatVec; ++v) {
+    for (int v = 0; v < VEC; ++v) {
         const long long i = i0 + 128 * v;
         whole[v] = i >= 0 && i + 4 <= n;
         if (whole[v]) {
@@ -1452,13 +1457,13 @@ __device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* 
         }
     }
 #pragma unroll
-    for (int k = 0; k < 4 * kFlatVec; ++k) p[k] = x[k] >= 0 ? __ldca(L + x[k]) : -1;
+    for (int k = 0; k < 4 * VEC; ++k) p[k] = x[k] >= 0 ? __ldca(L + x[k]) : -1;
     // one hop of every unfinished walk per round, their loads together
     bool more;
     do {
         more = false;
 #pragma unroll
-        for (int k = 0; k < 4 * kFlatVec; ++k)
+        for (int k = 0; k < 4 * VEC; ++k)
             if (p[k] != x[k]) {
                 x[k] = p[k];
                 p[k] = __ldca(L + x[k]);
@@ -1466,7 +1471,7 @@ __device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* 
             }
     } while (more);
 #pragma unroll
-    for (int v = 0; v < kFlatVec; ++v) {
+    for (int v = 0; v < VEC; ++v) {
         const long long i = i0 + 128 * v;
         if (whole[v]) {
             *reinterpret_cast<int4*>(L + i) = make_int4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
@@ -1493,7 +1498,7 @@ __device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* 
         int first = -1, mine = 0;
         bool one = true;
 #pragma unroll
-        for (int k = 0; k < 4 * kFlatVec; ++k) {
+        for (int k = 0; k < 4 * VEC; ++k) {
             if (x[k] < 0) continue;
             if (first < 0) first = x[k];
             one &= x[k] == first;
@@ -1508,7 +1513,7 @@ __device__ __forceinline__ void flatten_block(int32_t* L, long long n, int32_t* 
             if (lane == lead) atomicAdd(sizes + root, count);
         } else {
 #pragma unroll
-            for (int k = 0; k < 4 * kFlatVec; ++k) {
+            for (int k = 0; k < 4 * VEC; ++k) {
                 const unsigned peers = __match_any_sync(0xffffffffu, x[k]);
                 if (x[k] >= 0 && lane == __ffs(peers) - 1) atomicAdd(sizes + x[k], __popc(peers));
             }
@@ -1521,12 +1526,12 @@ __device__ __forceinline__ void flatten_phase(const FrameArgs& a) {
     int32_t* const L = a.labels;
     int32_t* const sizes = a.sizes;
     int32_t* const copy = sizes ? nullptr : a.labels_copy;   // with tri_min the filter writes it
-    const long long blocks = flatten_blocks(n);
+    const long long blocks = flatten_blocks<kFlatVec>(n);
     const int warps = gridDim.x * (kThreads / 32);
     // warp k of every CTA takes blocks k gridDim.x + the CTA's index: a frame of fewer blocks than
     // warps spreads over all SMs
     for (long long b = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; b < blocks; b += warps)
-        flatten_block(L, n, sizes, copy, b);
+        flatten_block<kFlatVec>(L, n, sizes, copy, b);
 }
 
 // Algorithm 5 keeps a segment only when it has more than tri_min triangles.
@@ -1787,16 +1792,17 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
     mark(2);
     {
         // every grouped triangle takes its root, block by block. Frame f's blocks start at
-        // tris[f] / kFlatBlock + 2 f: at least flatten_blocks() of them, the last ones empty
-        const long long total = __ldg(b.tris + n) / frame::kFlatBlock + 2LL * n;
+        // tris[f] / B + 2 f: at least flatten_blocks() of them, the last ones empty
+        constexpr int B = frame::kFlatBlock<frame::kFlatVecBatch>;
+        const long long total = __ldg(b.tris + n) / B + 2LL * n;
         int f = 0;
         for (long long k = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; k < total;
              k += (long long)gridDim.x * (kThreads / 32)) {
-            while (__ldg(b.tris + f + 1) / frame::kFlatBlock + 2LL * (f + 1) <= k) ++f;
+            while (__ldg(b.tris + f + 1) / B + 2LL * (f + 1) <= k) ++f;
             const long long t0 = __ldg(b.tris + f);
             const FrameArgs& a = b.frames[f];
-            frame::flatten_block(a.labels, __ldg(b.tris + f + 1) - t0, a.sizes, nullptr,
-                                 k - (t0 / frame::kFlatBlock + 2LL * f));
+            frame::flatten_block<frame::kFlatVecBatch>(a.labels, __ldg(b.tris + f + 1) - t0, a.sizes, nullptr,
+                                                       k - (t0 / B + 2LL * f));
         }
     }
     if (any_filter) {
