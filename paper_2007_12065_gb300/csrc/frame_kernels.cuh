@@ -1007,7 +1007,8 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     // runs' parents. What bounds it is latency: short dependent steps on two CTAs per SM. The label
     // stage took 7.4 us of a tile's 26 us in a 256-frame batch with prefix-max shuffles for the
     // runs, a compare-and-swap union per linked pair of runs and a walk per run, and takes 5.5 us
-    // with ballots and rounds over all links at once (batch 5869 -> 5716 us; 64 frames at one
+    // with ballots and rounds over all links at once, 4.7 us with the links inside a warp made on the
+    // way down its rows (batch 5869 -> 5716 us at the first; 64 frames at one
     // iteration 916 -> 882 us; a 480x640 frame 69.6 -> 68.1 us).
     //
     // free after the last iteration (>= 6 * nqs floats, nqs >= (TH + 1) T): parents of the run
@@ -1118,14 +1119,33 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     auto group_of = [&](int k) { return (int)(grp >> (8 * k)) & 255; };   // 2 row + side
     // (1) Runs along each quad row. Chain position 2v is second(v), 2v+1 is first(v); a run breaks
     // at second(v) unless first(v-1) links to it (right), at first(v) unless the quad's diagonal
-    // links (diag). The last break at or before a position comes from the two ballots.
-    int repF[kRows], repS[kRows];                        // run representatives, -1 without a group
-    unsigned bD[kRows], bR[kRows];
+    // links (diag). The last break at or before a position comes from the two ballots. A run linked to
+    // one of the warp's row above takes that run's root at its first link, so that what is left for
+    // the rounds below is a forest of few roots and shallow chains.
+    int rootF[kRows], rootS[kRows];                      // roots inside the warp's rows, -1 without a group
+    unsigned bD[kRows] = {}, bR[kRows] = {};
+    int x[kRows], y[kRows];                              // the ends of links still to make; equal: none
+    bool own[2 * kRows];                                 // this triangle is a root
     const unsigned le = kFull >> (31 - lane), lt = le >> 1;
+    // first(r, v) with second(r-1, v), of group g_up: the lanes that link, without those whose runs,
+    // above and below, both reach from the link of their left neighbour
+    auto links = [&](int row, int g_up, unsigned upD, unsigned upR, unsigned& all) {
+        const int r = r0 + row, gf = group_of(2 * row);
+        bool link = gf != PL3D_NO_GROUP && g_up == gf;
+        if (offs && link) {
+            V3 cf, c1, c0u, cu;
+            load_quad(Cq, (r + h) * RQW + (lane + h), cf, c1);
+            load_quad(Cq, (r - 1 + h) * RQW + (lane + h), c0u, cu);
+            link = offset_ok(gf, cf, cu);
+        }
+        all = __ballot_sync(kFull, link);
+        return all & ~((all << 1) & (bR[row] << 1) & bD[row] & (upD << 1) & (upR << 1));
+    };
 #pragma unroll
     for (int row = 0; row < kRows; ++row) {
-        repF[row] = repS[row] = -1;
-        bD[row] = bR[row] = 0;
+        rootF[row] = rootS[row] = -1;
+        x[row] = y[row] = 0;
+        own[2 * row] = own[2 * row + 1] = false;
         if (row >= rows) continue;
         const int r = r0 + row;
         const int gf = group_of(2 * row), gs = group_of(2 * row + 1);
@@ -1153,12 +1173,34 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
             return 2 * (r * T + l0) + (((p & 1) || !((brk_f >> l0) & 1u)) ? 0 : 1);
         };
         const int tf = 2 * (r * T + lane);
-        if (gf != PL3D_NO_GROUP) repF[row] = root_of(start_f);
-        if (gs != PL3D_NO_GROUP) repS[row] = root_of(start_s);
-        if (repF[row] == tf) Lp[tf] = tf;
-        if (repS[row] == tf + 1) Lp[tf + 1] = tf + 1;
+        if (gf != PL3D_NO_GROUP) rootF[row] = root_of(start_f);
+        if (gs != PL3D_NO_GROUP) rootS[row] = root_of(start_s);
+        if (row > 0) {
+            unsigned all;
+            const unsigned some = links(row, group_of(row > 0 ? 2 * row - 1 : 0), bD[row > 0 ? row - 1 : 0],
+                                        bR[row > 0 ? row - 1 : 0], all);
+            // the lanes whose first triangle is in this lane's run: from the run's start to its last
+            const unsigned cont = bR[row] & (bD[row] >> 1);        // first(v) reaches first(v+1)
+            const int last = lane + __ffs((int)~(cont >> lane)) - 1;
+            const unsigned run = (kFull >> (31 - last)) & (kFull << (start_f >> 1));
+            const int f = __ffs((int)(all & run)) - 1;             // the run's first link
+            const int up = rootS[row > 0 ? row - 1 : 0];
+            const int root = __shfl_sync(kFull, up, f & 31);
+            if (gf != PL3D_NO_GROUP && f >= 0) rootF[row] = root;
+            const int left = __shfl_up_sync(kFull, rootF[row], 1);
+            if (diag) rootS[row] = rootF[row];
+            else if (lane > 0 && ((bR[row] >> (lane - 1)) & 1u)) rootS[row] = left;
+            if (((some >> lane) & 1u) && up != rootF[row]) {
+                x[row] = rootF[row];
+                y[row] = up;
+            }
+        }
+        own[2 * row] = rootF[row] == tf;
+        own[2 * row + 1] = rootS[row] == tf + 1;
+        if (own[2 * row]) Lp[tf] = tf;
+        if (own[2 * row + 1]) Lp[tf + 1] = tf + 1;
         if (row == rows - 1) {
-            UpRep[threadIdx.x] = repS[row];
+            UpRep[threadIdx.x] = rootS[row];
             UpGrp[threadIdx.x] = gs;
             if (lane == 0) {
                 UpMask[2 * warp] = bD[row];
@@ -1167,59 +1209,45 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
         }
     }
     __syncthreads();
-    // (2) Rows joined across horizontal edges: first(r, v) with second(r-1, v). A lane whose runs,
-    // above and below, both reach from the link of its left neighbour leaves the link to it.
-    int repU[kRows];
-    unsigned todo = 0;                                   // this thread's links not yet inside one segment
-#pragma unroll
-    for (int row = 0; row < kRows; ++row) {
-        repU[row] = -1;
-        if (row >= rows || (row == 0 && warp == 0)) continue;
-        const int r = r0 + row;
-        const int g_up = row == 0 ? UpGrp[threadIdx.x - 32] : group_of(row > 0 ? 2 * row - 1 : 0);
-        const unsigned upD = row == 0 ? UpMask[2 * warp - 2] : bD[row > 0 ? row - 1 : 0];
-        const unsigned upR = row == 0 ? UpMask[2 * warp - 1] : bR[row > 0 ? row - 1 : 0];
-        repU[row] = row == 0 ? UpRep[threadIdx.x - 32] : repS[row > 0 ? row - 1 : 0];
-        const int gf = group_of(2 * row);
-        bool link = gf != PL3D_NO_GROUP && g_up == gf;
-        if (offs && link) {
-            V3 cf, c1, c0u, cu;
-            load_quad(Cq, (r + h) * RQW + (lane + h), cf, c1);
-            load_quad(Cq, (r - 1 + h) * RQW + (lane + h), c0u, cu);
-            link = offset_ok(gf, cf, cu);
+    // (2) The links of the warp's first row with the row above, another warp's.
+    if (warp > 0) {
+        unsigned all;
+        const unsigned some = links(0, UpGrp[threadIdx.x - 32], UpMask[2 * warp - 2], UpMask[2 * warp - 1], all);
+        if ((some >> lane) & 1u) {
+            x[0] = rootF[0];
+            y[0] = UpRep[threadIdx.x - 32];
         }
-        const unsigned bL = __ballot_sync(kFull, link);
-        const unsigned same = (bL << 1) & (bR[row] << 1) & bD[row] & (upD << 1) & (upR << 1);
-        if (link && !((same >> lane) & 1u)) todo |= 1u << row;
     }
     // (3) Segments from the links, in rounds over all links at once. At the start of a round every
-    // representative points at its root. A link between two roots lowers the parent of the larger
+    // root of (1) points at its root so far. A link between two roots lowers the parent of the larger
     // to the smaller (the smallest wins; a link stays on the list until it finds its two ends under
-    // one root, so one whose update lost is tried again). Then each representative jumps to its root,
+    // one root, so one whose update lost is tried again). Then each root of (1) jumps to its root,
     // all at once, which takes the logarithm of a chain's length. A round that changes anything removes
     // a root; scans take two or three rounds.
     // A thread's loads are issued together in every step: what bounds a round is their latency.
     volatile int32_t* const vp = Lp;
     while (true) {
-        int x[kRows], y[kRows];
+        int a0[kRows], b0[kRows];
+        bool todo = false;
 #pragma unroll
         for (int row = 0; row < kRows; ++row) {
-            const bool on = (todo >> row) & 1u;
-            x[row] = on ? vp[repF[row]] : 0;
-            y[row] = on ? vp[repU[row]] : 0;
+            const bool on = x[row] != y[row];
+            a0[row] = on ? vp[x[row]] : 0;
+            b0[row] = on ? vp[y[row]] : 0;
         }
 #pragma unroll
         for (int row = 0; row < kRows; ++row) {
-            if (x[row] != y[row]) atomicMin(Lp + max(x[row], y[row]), min(x[row], y[row]));
-            else todo &= ~(1u << row);
+            if (a0[row] != b0[row]) {
+                atomicMin(Lp + max(a0[row], b0[row]), min(a0[row], b0[row]));
+                todo = true;
+            } else {
+                x[row] = y[row];
+            }
         }
-        if (!__syncthreads_or(todo != 0)) break;
-        int up[2 * kRows];                               // current parent of each own representative, -1: none
+        if (!__syncthreads_or(todo)) break;
+        int up[2 * kRows];                               // current parent of each own root, -1: none
 #pragma unroll
-        for (int k = 0; k < 2 * kRows; ++k) {
-            const int t = 2 * ((r0 + (k >> 1)) * T + lane) + (k & 1);
-            up[k] = ((k & 1) ? repS[k >> 1] : repF[k >> 1]) == t ? vp[t] : -1;   // (a row past the warp's: -1)
-        }
+        for (int k = 0; k < 2 * kRows; ++k) up[k] = own[k] ? vp[2 * ((r0 + (k >> 1)) * T + lane) + (k & 1)] : -1;
         bool more;
         do {
             more = false;
@@ -1244,7 +1272,7 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
     for (int row = 0; row < kRows; ++row) {
         if (row >= rows) break;
         const int gu = ty * TH + r0 + row;
-        const int tF = repF[row] >= 0 ? Lp[repF[row]] : -1, tS = repS[row] >= 0 ? Lp[repS[row]] : -1;
+        const int tF = rootF[row] >= 0 ? Lp[rootF[row]] : -1, tS = rootS[row] >= 0 ? Lp[rootS[row]] : -1;
         // tile-local index 2 (row T + column) + side -> GID
         const int labF = tF >= 0 ? base + (tF / (2 * T)) * (2 * Wq) + tF % (2 * T) : -1;
         const int labS = tS >= 0 ? base + (tS / (2 * T)) * (2 * Wq) + tS % (2 * T) : -1;
