@@ -662,7 +662,10 @@ __device__ __forceinline__ V3 own_sum(const OwnTri& o) {
     return {a + b, c + d, e + f};
 }
 
-// A quad's two triangles: their own quad first (each triangle's weight with itself is exactly 1).
+// A quad's two triangles: their own quad first. Each triangle's weight with itself is exactly 1, so what
+// is left is one weight of each with the other, in scalar steps that share the difference of the
+// centroids (the same roundings as a half of own_weights): 21 FP32 cycles instead of 48 of a quad's 432,
+// a packed instruction taking two. 480x640 frame 64.4 -> 64.0 us, 256 frames 5012 -> 4969 us.
 struct QuadAcc {
     OwnTri t0, t1;
     V3 n0, n1;   // current normals (a triangle without a normal keeps n = 0)
@@ -683,10 +686,16 @@ __device__ __forceinline__ void quad_begin(QuadAcc& A, const float* Cq, const fl
     A.n1 = {n1x, n1y, n1z};
     own_begin(A.t0, {c0x, c0y, c0z}, A.n0, a);
     own_begin(A.t1, {c1x, c1y, c1z}, A.n1, a);
-    const f2 w0 = own_weights(A.t0, a2, cx, cy, cz, nx, ny, nz);
-    own_add(A.t0, pk(1.f, hi_of(w0)), nx, ny, nz);
-    const f2 w1 = own_weights(A.t1, a2, cx, cy, cz, nx, ny, nz);
-    own_add(A.t1, pk(lo_of(w1), 1.f), nx, ny, nz);
+    const float dx = c0x - c1x, dy = c0y - c1y, dz = c0z - c1z;
+    float e0 = fmaf(lo_of(A.t0.px), n1x, a), e1 = fmaf(lo_of(A.t1.px), n0x, a);
+    e0 = fmaf(lo_of(A.t0.py), n1y, e0), e1 = fmaf(lo_of(A.t1.py), n0y, e1);
+    e0 = fmaf(lo_of(A.t0.pz), n1z, e0), e1 = fmaf(lo_of(A.t1.pz), n0z, e1);
+    e0 = fmaf(dz, dz, e0), e1 = fmaf(dz, dz, e1);
+    e0 = fmaf(dy, dy, e0), e1 = fmaf(dy, dy, e1);
+    e0 = fmaf(dx, dx, e0), e1 = fmaf(dx, dx, e1);
+    const float w0 = ex2(-e0), w1 = ex2(-e1);
+    A.t0.sx = pk(n0x, w0 * n1x), A.t0.sy = pk(n0y, w0 * n1y), A.t0.sz = pk(n0z, w0 * n1z);
+    A.t1.sx = pk(w1 * n0x, n1x), A.t1.sy = pk(w1 * n0y, n1y), A.t1.sz = pk(w1 * n0z, n1z);
 }
 
 __device__ __forceinline__ void quad_neighbour(QuadAcc& A, f2 a2, f2 cx, f2 cy, f2 cz, f2 nx, f2 ny, f2 nz) {
