@@ -671,7 +671,7 @@ struct QuadAcc {
     V3 n0, n1;   // current normals (a triangle without a normal keeps n = 0)
 };
 
-__device__ __forceinline__ void quad_begin(QuadAcc& A, const float* Cq, const float* cur, int q, float a, f2 a2) {
+__device__ __forceinline__ void quad_begin(QuadAcc& A, const float* Cq, const float* cur, int q, float a) {
     f2 cx, cy, cz, nx, ny, nz;
     load_quad2(Cq, q, cx, cy, cz);
     load_quad2(cur, q, nx, ny, nz);
@@ -963,8 +963,8 @@ __device__ void bil_tile(const FrameArgs& a, const BilPhase& ph, int tile, float
             const bool two = qr + 1 < RQH - lo;
             const int qA = qr * RQW + qc, qB = qA + RQW;
             QuadAcc A, B;
-            quad_begin(A, Cq, cur, qA, an, a2);
-            quad_begin(B, Cq, cur, qB, an, a2);
+            quad_begin(A, Cq, cur, qA, an);
+            quad_begin(B, Cq, cur, qB, an);
 #pragma unroll
             for (int dr = -R; dr <= R + 1; ++dr) {
 #pragma unroll
