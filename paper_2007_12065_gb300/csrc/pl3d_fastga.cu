@@ -478,15 +478,16 @@ __device__ __forceinline__ int ga_bin(const GaArgs& a, float x, float y, float z
     return by * a.grid + bx;
 }
 
-// The cell of a point whose bin holds `place`.
-__device__ __forceinline__ int ga_cell(const GaArgs& a, const GaPoint& g, int place) {
+// The cell of a point whose bin holds `place`, and `k`, the first cell that a bin of several keeps.
+__device__ __forceinline__ const float4* ga_kept(const GaArgs& a, int place) { return a.multi + ((-1 - place) >> 4); }
+
+__device__ __forceinline__ int ga_cell(const GaArgs& a, const GaPoint& g, int place, float4 k) {
     if (place < 0) {
-        const int code = -1 - place;
-        const float4* m = a.multi + (code >> 4);
-        float4 k = __ldg(m);
+        const int count = (-1 - place) & 15;
+        const float4* m = ga_kept(a, place);
         float bd = g.t * k.x + g.u * k.y + g.v * k.z;
         place = __float_as_int(k.w);
-        for (int o = 1; o < (code & 15); ++o) {
+        for (int o = 1; o < count; ++o) {
             k = __ldg(m + o);
             const float dd = g.t * k.x + g.u * k.y + g.v * k.z;
             if (dd > bd) {
@@ -502,10 +503,11 @@ constexpr int kGaThreads = 512;
 constexpr int kGaBatch = 4;   // normals a thread loads before it locates them
 
 // One cooperative launch. What bounds it is latency: a normal's load, its bin's, the bin's cells', one
-// after another, and the grid barrier. Every CTA clears its share of the output histogram and
-// arrives at the barrier at once, so that its opening is long past when the CTA waits for it; then each
-// thread loads kGaBatch normals (a 480x640 frame's triangles in one round over the chip), reads their
-// bins together, and counts them in the CTA's private histogram, which is added to the output
+// after another, and the grid barrier. Every CTA clears its share of the output histogram, issues the loads
+// of its first normals and arrives at the barrier, so that its opening is long past when the CTA waits
+// for it. A thread takes kGaBatch normals at a time (a 480x640 frame's triangles in one round over the
+// chip), each of the three steps' loads of all of them together, and counts them in
+// the CTA's private histogram, which is added to the output
 // after the barrier. 480x640: 14.3 -> 13.6 us against two rounds of two normals and a whole barrier.
 __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_constant__ GaArgs a) {
     extern __shared__ int hist[];   // [cells]
@@ -515,39 +517,44 @@ __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_cons
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.cells;
          i += (long long)gridDim.x * blockDim.x)
         a.counts[i] = 0;
-    grid_barrier_arrive(a.barrier, &gen);   // (its CTA barrier also publishes the cleared histogram)
     const long long n_samples = a.n_samples;
     const long long T = (long long)gridDim.x * blockDim.x;
     const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     for (long long it = 0; it < a.n_iter; ++it) {
         float x[kGaBatch], y[kGaBatch], z[kGaBatch];
-        bool ok[kGaBatch];
+        uint8_t used[kGaBatch];
         const long long s0 = g + kGaBatch * it * T;   // the batch's samples: s0 + k T
 #pragma unroll
         for (int k = 0; k < kGaBatch; ++k) {
             const long long s = s0 + k * T;
             x[k] = y[k] = z[k] = NAN;
-            ok[k] = s < n_samples;
-            if (ok[k]) {
+            used[k] = s < n_samples;
+            if (used[k]) {
                 const long long i = s * a.stride;
                 x[k] = __ldg(a.normals + 3 * i);
                 y[k] = __ldg(a.normals + 3 * i + 1);
                 z[k] = __ldg(a.normals + 3 * i + 2);
-                ok[k] = !a.mask || __ldg(a.mask + i) != 0;
+                if (a.mask) used[k] = __ldg(a.mask + i);
             }
         }
+        if (it == 0) grid_barrier_arrive(a.barrier, &gen);   // (its CTA barrier also publishes the cleared histogram)
         GaPoint pt[kGaBatch];
         int place[kGaBatch];
+        bool ok[kGaBatch];
 #pragma unroll
         for (int k = 0; k < kGaBatch; ++k) {
-            ok[k] = ok[k] && isfinite(x[k]) && isfinite(y[k]) && isfinite(z[k]);
+            ok[k] = used[k] && isfinite(x[k]) && isfinite(y[k]) && isfinite(z[k]);
             place[k] = 0;
             if (ok[k]) place[k] = __ldg(a.bins + ga_bin(a, x[k], y[k], z[k], pt[k]));
         }
+        float4 kept[kGaBatch];
+#pragma unroll
+        for (int k = 0; k < kGaBatch; ++k)
+            if (place[k] < 0) kept[k] = __ldg(ga_kept(a, place[k]));
 #pragma unroll
         for (int k = 0; k < kGaBatch; ++k) {
-            const int cell = ok[k] ? ga_cell(a, pt[k], place[k]) : -1;
+            const int cell = ok[k] ? ga_cell(a, pt[k], place[k], kept[k]) : -1;
             // the warp's first counted cell in one shared-memory atomic, the lanes of other cells
             // one each (neighbouring triangles mostly share a cell)
             const unsigned counted = __ballot_sync(0xffffffffu, cell >= 0);
