@@ -1680,11 +1680,11 @@ __device__ __forceinline__ int find_frame(const int* pre, int n, int t) {
     return lo;
 }
 
-// Tiles of a batch phase go to the CTAs in runs of kRun consecutive tiles, dealt round-robin.
-constexpr int kRun = 4;
-__device__ __forceinline__ int next_tile(int t) {
-    return (t + 1) % kRun != 0 ? t + 1 : (t / kRun + (int)gridDim.x) * kRun;
-}
+// Tiles of a batch phase go to the CTAs one at a time, round-robin, so that no CTA gets more than one
+// above the others: in runs of 4 consecutive tiles (closer halos, a tensor-map acquire per run) a CTA
+// took 8 tiles of a batch that has 4.5 for each, 368 us for 8 mixed frames against 254 us, 1014 / 977 for
+// 48, 5465 / 5352 for 256 of one mix (one iteration: 209 / 156, 576 / 557, 3109 / 3080).
+__device__ __forceinline__ int next_tile(int t) { return t + (int)gridDim.x; }
 
 // Advances f (never backwards) to the frame whose range of pre holds item i.
 __device__ __forceinline__ int advance_frame(const long long* pre, int f, long long i) {
@@ -1745,10 +1745,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
             }
             frame::lap_issue(a, a.lap[c], map, t - __ldg(pre + f), smem + slot * P, bar + slot);
         };
-        // runs of kRun consecutive tiles dealt round-robin: neighbouring tiles, whose halos
-        // overlap, close together in time, a map acquire per run, and the balance of a
-        // round-robin when frames differ in cost
-        const int t_begin = (int)blockIdx.x * frame::kRun;
+        const int t_begin = (int)blockIdx.x;
         int f_cur = t_begin < total ? frame::find_frame(pre, n, t_begin) : 0;
         // the furthest tile of the sequence issued so far, and its frame (frames grow along it)
         int t_ahd = t_begin, f_ahd = f_cur;
@@ -1788,7 +1785,7 @@ __global__ void __launch_bounds__(kThreads, 2) batch_kernel(const __grid_constan
         const int* pre = b.bil_tiles + c * b.stride;
         const int total = __ldg(pre + n);
         int acquired = -1;   // frames come in increasing order: each frame's maps acquired once
-        const int t_begin = (int)blockIdx.x * frame::kRun;
+        const int t_begin = (int)blockIdx.x;
         int f = t_begin < total ? frame::find_frame(pre, n, t_begin) : 0;
         for (int t = t_begin; t < total; t = frame::next_tile(t)) {
             while (__ldg(pre + f + 1) <= t) ++f;
