@@ -333,8 +333,8 @@ int pl3d_extract_planes_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, 
  *                Either depth is raised where needed so that a filter takes at most 8 passes.
  *   ctas_per_sm  resident CTAs per SM of the persistent launch (0 = as many as fit, at most 2).
  *   lap_tile_h   Laplacian tile height in points, a multiple of 8 in [16, 64] (0 = by the frame's
- *                size for a single frame; 32 in a batch, or 64 for a single-iteration first
- *                pass); tiles are 32 points wide. A height whose buffers would not fit two CTAs
+ *                size for a single frame; 32 in a batch, or 64 where it fits with a 3 x 3 window
+ *                and for a single-iteration first pass); tiles are 32 points wide. A height whose buffers would not fit two CTAs
  *                per SM for a pass falls back to 32 for that pass.
  *   bil_tile_h   bilateral tile height in quads, a multiple of 8 in [8, 32] (0 = by the frame's
  *                size for a single frame, 32 in a batch); tiles are 32 quads wide (a warp labels

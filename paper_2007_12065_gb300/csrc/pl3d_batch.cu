@@ -191,11 +191,12 @@ int check_frames(const pl3d_frame* frames, int n, int* rl_out, int* rb_out) {
 }
 
 // Whether a batch with a 3 x 3 window whose tuning leaves it open runs its Laplacian as one iteration per
-// pass (lap1_kernel). Its warps walk 24 rows each, so a pass takes a round of them however few there
-// are; from 1.5 rounds over the chip on, five passes of 24-36 bytes a point take less than one
-// fused pass with its halos (mixed frames, 2 / 3 / 5 iterations: 8.5 M points 1154 / 1247 / 1396 ->
-// 1125 / 1221 / 1345 us, 37 M points 5615 -> 5271 us; 5.8 M points, just above the line, 836 / 898 / 998 ->
-// 832 / 907 / 981 us; 4 M points 726 -> 745 us at 5 iterations). Every frame has to fit kMaxPasses.
+// pass (lap1_kernel) instead of one fused pass of tiles, 64 rows high where they fit. A warp of that
+// kernel walks 24 rows, so a pass takes a round of them however few there are; from 3 rounds over the
+// chip on (about 11 M points), five passes of 24-36 bytes a point take less than one fused pass with
+// its halos (mixed frames at 5 / 2 iterations, us: 3.7 rounds 1863 / 1557 against 1907 / 1575, 5.4 rounds
+// 2676 / 2236 against 2773 / 2270; below it 2.4 rounds 1235 / 1022 against 1207 / 1023, 1.3 rounds 735 /
+// 611 against 665 / 578; with 32-row tiles 687 / 586). Every frame has to fit kMaxPasses.
 bool single_passes(const pl3d_frame* frames, int n, int dev) {
     long long tasks = 0;
     for (int i = 0; i < n; ++i) {
@@ -203,7 +204,7 @@ bool single_passes(const pl3d_frame* frames, int n, int dev) {
         tasks += lap1_tasks(frames[i].H, frames[i].W);
     }
     const long long warps = (long long)lap1_grid(dev, true, -1) * (kLap1Threads / 32);
-    return warps > 0 && 2 * tasks >= 3 * warps;
+    return warps > 0 && tasks >= 3 * warps;
 }
 
 int run_batch(pl3d_ctx* c, const pl3d_frame* frames, int n, cudaStream_t s) {
@@ -211,8 +212,10 @@ int run_batch(pl3d_ctx* c, const pl3d_frame* frames, int n, cudaStream_t s) {
     int rc = check_frames(frames, n, &rl, &rb);
     if (rc != PL3D_OK || n == 0) return rc;
     Tuning t = c->tuning;
-    if (t.lap_fuse == 0 && t.lap_tile_h == 0 && t.ctas_per_sm == 0 && rl == 1 && single_passes(frames, n, c->device))
-        t.lap_fuse = 1;
+    if (t.lap_fuse == 0 && t.lap_tile_h == 0 && t.ctas_per_sm == 0 && rl == 1) {
+        if (single_passes(frames, n, c->device)) t.lap_fuse = 1;
+        else t.lap_tile_h = kLapMaxTileH;
+    }
 
     size_t slab = 0;
     for (int i = 0; i < n; ++i) slab += frame_needs(frames[i], t).total();

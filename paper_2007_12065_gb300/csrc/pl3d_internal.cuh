@@ -241,7 +241,8 @@ struct Tuning {
     int bil_fuse;                  // same for the bilateral
     int ctas_per_sm;               // 0 = as many as fit
     int lap_tile_h;                // Laplacian tile height in points, 0 = by frame_tuning for a single
-                                   // frame, 32 in a batch (64 for a single-iteration first pass); a
+                                   // frame, 32 in a batch (64 with a 3 x 3 window and for a
+                                   // single-iteration first pass); a
                                    // height whose buffers would not fit two CTAs per SM falls back to 32
     int bil_tile_h;                // bilateral tile height in quads, 0 = by frame_tuning for a single
                                    // frame, 32 in a batch
