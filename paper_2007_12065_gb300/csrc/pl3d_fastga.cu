@@ -449,8 +449,7 @@ struct GaArgs {
 //     cells the bin keeps.
 //  4. That cell in face f0's frame: face 0's cell c is face f0's cell f0 4^level + c, a cell of
 //     the 1-ring outside face 0 is looked up.
-// Steps 1 and 2 (ga_bin) come before the table reads of 3 and 4 (ga_cell), so that a thread's bins are
-// all on their way before it needs the first.
+// Steps 1 and 2 are ga_bin, the bin's cell or the search over its cells and step 4 are ga_cell.
 struct GaPoint {
     int f0;
     float t, u, v;
@@ -500,15 +499,20 @@ __device__ __forceinline__ int ga_cell(const GaArgs& a, const GaPoint& g, int pl
 }
 
 constexpr int kGaThreads = 512;
-constexpr int kGaBatch = 4;   // normals a thread loads before it locates them
+constexpr int kGaBatch = 2;   // normals a thread loads before it locates them
 
-// One cooperative launch. What bounds it is latency: a normal's load, its bin's, the bin's cells', one
-// after another, and the grid barrier. Every CTA clears its share of the output histogram, issues the loads
-// of its first normals and arrives at the barrier, so that its opening is long past when the CTA waits
-// for it. A thread takes kGaBatch normals at a time (a 480x640 frame's triangles in one round over the
-// chip), each of the three steps' loads of all of them together, and counts them in
-// the CTA's private histogram, which is added to the output
-// after the barrier. 480x640: 14.3 -> 13.6 us against two rounds of two normals and a whole barrier.
+// One cooperative launch. Every CTA clears its share of the output histogram and arrives at the grid
+// barrier (every share cleared) before it locates any normal, so that the barrier's opening is long past
+// when the CTA waits for it. A thread takes kGaBatch normals at a time, loads them together and counts
+// them in the CTA's private histogram, which is added to the output after the barrier.
+//
+// What bounds a frame's call is latency (launch, a normal's load, its bin's, the bin's cells', one after
+// another); a large call is bound by instruction issue, and by shared-memory atomics where a warp's
+// normals fall into many cells. Level 4, us, against a whole barrier after the loop: 611,000 normals about
+// one direction 14.5 -> 12.5, of all directions 33.3 -> 28.1; 1,837,000 24.9 -> 22.9 and 76.2 -> 70.0;
+// 12 million 126.6 -> 119.0 and 416 -> 418. Four normals per thread, their bins and then their first
+// kept cells read together: 12.7 and 31.0, 26.1 and 76.2, 140 and 462: the steps of one normal
+// overlap less with another's, and registers spill.
 __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_constant__ GaArgs a) {
     extern __shared__ int hist[];   // [cells]
     __shared__ unsigned gen;
@@ -517,44 +521,39 @@ __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_cons
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.cells;
          i += (long long)gridDim.x * blockDim.x)
         a.counts[i] = 0;
+    grid_barrier_arrive(a.barrier, &gen);   // (its CTA barrier also publishes the cleared histogram)
     const long long n_samples = a.n_samples;
     const long long T = (long long)gridDim.x * blockDim.x;
     const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     for (long long it = 0; it < a.n_iter; ++it) {
         float x[kGaBatch], y[kGaBatch], z[kGaBatch];
-        uint8_t used[kGaBatch];
-        const long long s0 = g + kGaBatch * it * T;   // the batch's samples: s0 + k T
+        bool use[kGaBatch], in_range[kGaBatch];
+        long long idx[kGaBatch];
 #pragma unroll
         for (int k = 0; k < kGaBatch; ++k) {
-            const long long s = s0 + k * T;
+            const long long s = g + (kGaBatch * it + k) * T;
+            in_range[k] = s < n_samples;
+            idx[k] = in_range[k] ? s * a.stride : 0;
             x[k] = y[k] = z[k] = NAN;
-            used[k] = s < n_samples;
-            if (used[k]) {
-                const long long i = s * a.stride;
-                x[k] = __ldg(a.normals + 3 * i);
-                y[k] = __ldg(a.normals + 3 * i + 1);
-                z[k] = __ldg(a.normals + 3 * i + 2);
-                if (a.mask) used[k] = __ldg(a.mask + i);
+            if (in_range[k]) {
+                x[k] = __ldg(a.normals + 3 * idx[k]);
+                y[k] = __ldg(a.normals + 3 * idx[k] + 1);
+                z[k] = __ldg(a.normals + 3 * idx[k] + 2);
             }
+            use[k] = in_range[k] && (!a.mask || __ldg(a.mask + idx[k]) != 0);
         }
-        if (it == 0) grid_barrier_arrive(a.barrier, &gen);   // (its CTA barrier also publishes the cleared histogram)
-        GaPoint pt[kGaBatch];
-        int place[kGaBatch];
-        bool ok[kGaBatch];
 #pragma unroll
         for (int k = 0; k < kGaBatch; ++k) {
-            ok[k] = used[k] && isfinite(x[k]) && isfinite(y[k]) && isfinite(z[k]);
-            place[k] = 0;
-            if (ok[k]) place[k] = __ldg(a.bins + ga_bin(a, x[k], y[k], z[k], pt[k]));
-        }
-        float4 kept[kGaBatch];
-#pragma unroll
-        for (int k = 0; k < kGaBatch; ++k)
-            if (place[k] < 0) kept[k] = __ldg(ga_kept(a, place[k]));
-#pragma unroll
-        for (int k = 0; k < kGaBatch; ++k) {
-            const int cell = ok[k] ? ga_cell(a, pt[k], place[k], kept[k]) : -1;
+            const bool ok = use[k] && isfinite(x[k]) && isfinite(y[k]) && isfinite(z[k]);
+            int cell = -1;
+            if (ok) {
+                GaPoint pt;
+                const int place = __ldg(a.bins + ga_bin(a, x[k], y[k], z[k], pt));
+                float4 kept;
+                if (place < 0) kept = __ldg(ga_kept(a, place));
+                cell = ga_cell(a, pt, place, kept);
+            }
             // the warp's first counted cell in one shared-memory atomic, the lanes of other cells
             // one each (neighbouring triangles mostly share a cell)
             const unsigned counted = __ballot_sync(0xffffffffu, cell >= 0);
@@ -564,7 +563,7 @@ __global__ void __launch_bounds__(kGaThreads, 2) fastga_kernel(const __grid_cons
                 if (lane == __ffs(counted) - 1) atomicAdd(hist + lead, __popc(same));
                 else if (cell >= 0 && cell != lead) atomicAdd(hist + cell, 1);
             }
-            if (a.out_cell && s0 + k * T < n_samples) a.out_cell[(s0 + k * T) * a.stride] = cell;
+            if (a.out_cell && in_range[k]) a.out_cell[idx[k]] = cell;
         }
     }
     __syncthreads();                                   // this CTA's histogram is final
