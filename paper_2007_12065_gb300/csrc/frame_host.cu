@@ -180,11 +180,12 @@ static int lap_tile_h(int iters, bool first, int halo, int requested) {
 static int bil_tile_h(const Tuning& t) { return t.bil_tile_h > 0 ? t.bil_tile_h : kTile; }
 
 // Time of a phase of `tiles` tiles: rounds of two CTAs per SM (`paired` each), the last one cheaper
-// when it leaves each SM one CTA; with one CTA per SM, rounds of `alone`.
-static double phase_cost(long long tiles, int sms, int per_sm, double paired, double alone) {
+// when it leaves each SM one CTA; with one CTA per SM, rounds of `alone`. `crowded`: the launch has more
+// CTAs than SMs whatever this phase needs, so two of them share an SM from the first tiles on.
+static double phase_cost(long long tiles, int sms, int per_sm, bool crowded, double paired, double alone) {
     if (per_sm < 2) return (double)((tiles + sms - 1) / sms) * alone;
     const long long full = tiles / (2LL * sms), rest = tiles % (2LL * sms);
-    return (double)full * paired + (rest == 0 ? 0.0 : rest <= sms ? alone : paired);
+    return (double)full * paired + (rest == 0 ? 0.0 : rest <= sms && (full > 0 || !crowded) ? alone : paired);
 }
 
 // Tile heights of a single frame whose tuning leaves them open. A phase lasts as long as its
@@ -196,49 +197,67 @@ static double phase_cost(long long tiles, int sms, int per_sm, double paired, do
 // staging and geometry per staged row, iterations per row and iteration, groups and labels per
 // row; a tile alone on its SM takes 0.66 (bilateral) or 0.8
 // (Laplacian) of the time of each of two.
+//
+// Both phases run on one grid, that of the phase with more tiles, so the two heights are chosen
+// together: 228 Laplacian tiles of 16 rows put two CTAs on some SMs, and 114 bilateral tiles then take
+// as long as two on one SM (49x1800 at 8 / 5 iterations: 74.9 us at heights 16 and 24, 61.8 us at 32 and
+// 24; at 5 / 3 51.7 and 45.5 us). Not with larger Laplacian windows, whose times step with the strips of
+// a tile (7 x 7, 298x310: 46.0 us at 16 rows, 50.7 us at 24). A phase's CTAs per SM are taken from its own
+// shared memory: counted by the larger need of the two, frames of four and more bilateral
+// iterations took 16-row bilateral tiles and 3 to 12% longer.
 Tuning frame_tuning(const Tuning& t, int H, int W, const pl3d_params* p, int dev) {
     Tuning r = t;
     int sms = 0;
     if (H < 2 || W < 2 || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
         return r;
-    constexpr double kBilAlone = 0.66, kLapAlone = 0.8;
+    constexpr double kBilAlone = 0.66, kLapAlone = 0.8, kTie = 1e-6;
     const auto per_sm = [&](size_t smem) { return smem <= (size_t)kTwoCtaSmem && t.ctas_per_sm != 1 ? 2 : 1; };
-    if (t.bil_tile_h == 0) {
-        const int R = p->bil_iters > 0 ? p->bil_kernel / 2 : 1;
-        const int fuse = fused_iters(p->bil_iters, kBilMaxHalo / R, t.bil_fuse);
-        const int n = p->bil_iters < fuse ? p->bil_iters : fuse, h = n * R;
-        const double window = R == 1 ? 0.15 : R == 2 ? 0.36 : 0.7;
-        double best = 0.0;
-        for (int th = kBilMaxTileH; th >= kBilMinTileH; th -= 8) {
-            double paired = 6.7 + 0.216 * (th + 2 * h) * (kTile + 2 * h) / 38.0 + 0.16 * th;
-            for (int i = 1; i <= n; ++i)
-                paired += window * (th + 2 * (h - i * R)) * (kTile + 2 * (h - i * R)) / 34.0;
-            const long long tiles = (long long)div_up(H - 1, th) * div_up(W - 1, kTile);
-            const double c = phase_cost(tiles, sms, per_sm(bil_smem(h, th)), paired, kBilAlone * paired);
-            if (r.bil_tile_h == 0 || c < best) {
+
+    const int rb = p->bil_iters > 0 ? p->bil_kernel / 2 : 1;
+    const int bfuse = fused_iters(p->bil_iters, kBilMaxHalo / rb, t.bil_fuse);
+    const int nb = p->bil_iters < bfuse ? p->bil_iters : bfuse, hb = nb * rb;
+    const double bil_window = rb == 1 ? 0.15 : rb == 2 ? 0.36 : 0.7;
+    const int rl = p->lap_iters > 0 ? p->lap_kernel / 2 : 1;
+    const int lfuse = fused_iters(p->lap_iters, kLapMaxHalo / rl, t.lap_fuse);
+    const int nl = p->lap_iters < lfuse ? p->lap_iters : lfuse, hl = nl * rl;
+    const double lap_window = rl == 1 ? 0.06 : rl == 2 ? 0.14 : 0.28;
+    const bool lap_open = t.lap_tile_h == 0 && nl > 1;   // (a single-iteration pass keeps its own rule, lap_tile_h)
+
+    struct LapChoice {
+        int th;
+        long long tiles;
+        int per_sm;
+        double paired;
+    };
+    LapChoice laps[kLapMaxTileH / 8];
+    int n_laps = 0;
+    for (int th = lap_open ? kLapMinTileH : lap_tile_h(nl, true, hl, t.lap_tile_h); th <= kLapMaxTileH; th += 8) {
+        const size_t smem = lap_smem_for(lap_box_floats(hl, th), 1, lap_thin(nl, true) ? 1 : 2);
+        if (lap_open && th > kTile && smem > (size_t)kTwoCtaSmem) break;
+        double paired = 3.0;
+        for (int i = 1; i <= nl; ++i)
+            paired += lap_window * (th + 2 * (hl - i * rl)) * (kTile + 2 * (hl - i * rl)) / 36.0;
+        laps[n_laps++] = {th, (long long)div_up(H, th) * div_up(W, kTile), per_sm(smem), paired};
+        if (!lap_open) break;
+    }
+    double best = -1.0;
+    for (int th = kBilMaxTileH; th >= kBilMinTileH; th -= 8) {
+        if (t.bil_tile_h != 0 && th != t.bil_tile_h) continue;
+        double paired = 6.7 + 0.216 * (th + 2 * hb) * (kTile + 2 * hb) / 38.0 + 0.16 * th;
+        for (int i = 1; i <= nb; ++i)
+            paired += bil_window * (th + 2 * (hb - i * rb)) * (kTile + 2 * (hb - i * rb)) / 34.0;
+        const long long tiles = (long long)div_up(H - 1, th) * div_up(W - 1, kTile);
+        const int bil_sm = per_sm(bil_smem(hb, th));
+        for (int k = 0; k < n_laps; ++k) {
+            const LapChoice& l = laps[k];
+            const bool crowded = rl == 1 && lap_open && bil_sm == 2 && l.per_sm == 2 && std::max(tiles, l.tiles) > sms;
+            double c = phase_cost(tiles, sms, bil_sm, crowded, paired, kBilAlone * paired);
+            if (lap_open) c += phase_cost(l.tiles, sms, l.per_sm, crowded, l.paired, kLapAlone * l.paired);
+            // (equal: the taller of two tiles, which leaves fewer CTAs)
+            if (best < 0.0 || c < best - kTie || (lap_open && th == r.bil_tile_h && c < best + kTie)) {
                 best = c;
                 r.bil_tile_h = th;
-            }
-        }
-    }
-    if (t.lap_tile_h == 0) {
-        const int R = p->lap_iters > 0 ? p->lap_kernel / 2 : 1;
-        const int fuse = fused_iters(p->lap_iters, kLapMaxHalo / R, t.lap_fuse);
-        const int n = p->lap_iters < fuse ? p->lap_iters : fuse, h = n * R;
-        // (a single-iteration pass keeps its own rule, lap_tile_h)
-        const double window = R == 1 ? 0.06 : R == 2 ? 0.14 : 0.28;
-        double best = 0.0;
-        for (int th = kLapMinTileH; n > 1 && th <= kLapMaxTileH; th += 8) {
-            const size_t smem = lap_smem_for(lap_box_floats(h, th), 1, 2);
-            if (th > kTile && smem > (size_t)kTwoCtaSmem) break;
-            double paired = 3.0;
-            for (int i = 1; i <= n; ++i)
-                paired += window * (th + 2 * (h - i * R)) * (kTile + 2 * (h - i * R)) / 36.0;
-            const long long tiles = (long long)div_up(H, th) * div_up(W, kTile);
-            const double c = phase_cost(tiles, sms, per_sm(smem), paired, kLapAlone * paired);
-            if (r.lap_tile_h == 0 || c < best) {
-                best = c;
-                r.lap_tile_h = th;
+                if (lap_open) r.lap_tile_h = l.th;
             }
         }
     }
