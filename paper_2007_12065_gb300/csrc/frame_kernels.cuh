@@ -1653,7 +1653,12 @@ __global__ void __launch_bounds__(kThreads, 2) frame_kernel(const __grid_constan
         }
         frame::phase_mark(a, 1, t_prev);
     }
-    if (a.part == 1) return;
+    if (a.part == 1) {
+        // one bilateral pass after a Laplacian in kernels of its own: no barrier, and with fewer tiles
+        // than CTAs some CTAs come here at once
+        grid_barrier_unused();
+        return;
+    }
     if (!a.border) {   // else the bilateral tiles joined their borders
         frame::merge_phase(a);
         grid_barrier(a.barrier, a.error, gen);

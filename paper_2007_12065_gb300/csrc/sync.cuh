@@ -143,6 +143,12 @@ __device__ __forceinline__ void grid_barrier_begin(const unsigned* bar, unsigned
     if (threadIdx.x == 0) cp_async4(reinterpret_cast<float*>(gen), reinterpret_cast<const float*>(bar + kBarrierGen));
 }
 
+// At the end of a launch that may reach no barrier: the copy of grid_barrier_begin has landed before the CTA
+// gives its shared memory back.
+__device__ __forceinline__ void grid_barrier_unused() {
+    if (threadIdx.x == 0) cp_async_wait_all();
+}
+
 // The two halves of a barrier, for work that fits between them (a CTA that has arrived must wait
 // before it arrives again).
 __device__ __forceinline__ void grid_barrier_arrive(unsigned* bar, unsigned* gen) {
