@@ -327,15 +327,18 @@ int pl3d_extract_planes_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, 
  * changes a result bit: iterations split over more passes go through global memory as the same
  * FP32 values the fused form keeps in shared memory.
  *   lap_fuse     most Laplacian iterations fused into one tile pass (0 = as many as the tile's
- *                halo of 8 points allows, or one per pass for a large batch with a 3 x 3 window);
+ *                halo of 8 points allows, or one per pass for a large batch, see lap_tile_h);
  *                fewer means smaller halos but more passes.
  *   bil_fuse     the same for the bilateral (halo of 6 quads).
  *                Either depth is raised where needed so that a filter takes at most 8 passes.
  *   ctas_per_sm  resident CTAs per SM of the persistent launch (0 = as many as fit, at most 2).
- *   lap_tile_h   Laplacian tile height in points, a multiple of 8 in [16, 64] (0 = by the frame's
- *                size for a single frame; 32 in a batch, or 64 where it fits with a 3 x 3 window
- *                and for a single-iteration first pass); tiles are 32 points wide. A height whose buffers would not fit two CTAs
- *                per SM for a pass falls back to 32 for that pass.
+ *   lap_tile_h   Laplacian tile height in points, a multiple of 8 in [16, 64]; tiles are 32 points
+ *                wide. 0 = by the frame's size for a single frame, 64 for a single-iteration first
+ *                pass, else 32. A batch with 3 x 3 windows whose lap_fuse and lap_tile_h are both 0
+ *                and whose ctas_per_sm is not 1 runs one iteration per pass when it is large (from
+ *                about 11 million points, at most 8 iterations each) and asks for 64 rows otherwise.
+ *                A height whose buffers would not fit two CTAs per SM for a pass falls back to 32
+ *                for that pass.
  *   bil_tile_h   bilateral tile height in quads, a multiple of 8 in [8, 32] (0 = by the frame's
  *                size for a single frame, 32 in a batch); tiles are 32 quads wide (a warp labels
  *                whole tile rows).

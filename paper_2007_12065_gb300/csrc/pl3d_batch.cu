@@ -207,15 +207,22 @@ bool single_passes(const pl3d_frame* frames, int n, int dev) {
     return warps > 0 && tasks >= 3 * warps;
 }
 
+// The tuning a batch of Laplacian radius rl runs under: t with what it leaves open of the Laplacian's shape
+// chosen for these frames, unless t asks for one CTA per SM, where the rule was not measured.
+Tuning batch_tuning(const Tuning& t, const pl3d_frame* frames, int n, int rl, int dev) {
+    Tuning r = t;
+    if (t.lap_fuse == 0 && t.lap_tile_h == 0 && t.ctas_per_sm != 1 && rl == 1) {
+        if (single_passes(frames, n, dev)) r.lap_fuse = 1;
+        else r.lap_tile_h = kLapMaxTileH;
+    }
+    return r;
+}
+
 int run_batch(pl3d_ctx* c, const pl3d_frame* frames, int n, cudaStream_t s) {
     int rl = 1, rb = 1;
     int rc = check_frames(frames, n, &rl, &rb);
     if (rc != PL3D_OK || n == 0) return rc;
-    Tuning t = c->tuning;
-    if (t.lap_fuse == 0 && t.lap_tile_h == 0 && t.ctas_per_sm == 0 && rl == 1) {
-        if (single_passes(frames, n, c->device)) t.lap_fuse = 1;
-        else t.lap_tile_h = kLapMaxTileH;
-    }
+    const Tuning t = batch_tuning(c->tuning, frames, n, rl, c->device);
 
     size_t slab = 0;
     for (int i = 0; i < n; ++i) slab += frame_needs(frames[i], t).total();
