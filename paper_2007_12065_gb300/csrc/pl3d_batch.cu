@@ -474,10 +474,17 @@ int pl3d_autotune_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, void* 
         lap_iters = std::max(lap_iters, (int)frames[i].params->lap_iters);
         bil_iters = std::max(bil_iters, (int)frames[i].params->bil_iters);
     }
-    std::vector<Tuning> round1;
+    // The shape that the batch has untuned, written out, comes first: whatever is installed is no slower.
+    Tuning untuned = batch_tuning(Tuning{0, 0, 0, 0, 0}, frames, n, rl, ctx->device);
+    if (untuned.lap_fuse == 0) untuned.lap_fuse = std::max(1, std::min(lap_iters, kLapMaxHalo / rl));
+    untuned.bil_fuse = std::max(1, std::min(bil_iters, kBilMaxHalo / rb));
+    untuned.ctas_per_sm = 2;
+    std::vector<Tuning> round1{untuned};
     for (int lf : fuse_candidates(lap_iters, kLapMaxHalo / rl, rl == 1))
         for (int bf : fuse_candidates(bil_iters, kBilMaxHalo / rb))
-            for (int cps : {1, 2}) round1.push_back(Tuning{lf, bf, cps, 0, 0});
+            for (int cps : {1, 2})
+                if (untuned.lap_tile_h != 0 || lf != untuned.lap_fuse || bf != untuned.bil_fuse || cps != untuned.ctas_per_sm)
+                    round1.push_back(Tuning{lf, bf, cps, 0, 0});
 
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
@@ -515,8 +522,8 @@ int pl3d_autotune_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, void* 
             }
         }
     };
-    // stage 1: fused depths and CTAs per SM at the default tile shapes; stage 2: tile heights at
-    // the best of those (the default shape is stage 1's own entry)
+    // stage 1: the untuned shape, and fused depths and CTAs per SM at 32-row tiles; stage 2: tile heights
+    // at the best of those
     try_all(round1);
     if (rc == PL3D_OK) {
         std::vector<Tuning> round2;
@@ -526,7 +533,8 @@ int pl3d_autotune_batched(pl3d_ctx* ctx, const pl3d_frame* frames, int n, void* 
                 c.lap_tile_h = lh;
                 c.bil_tile_h = bh == kTile ? 0 : bh;
                 if (c.lap_tile_h == kTile) c.lap_tile_h = 0;
-                if (c.lap_tile_h != 0 || c.bil_tile_h != 0) round2.push_back(c);
+                if (c.lap_tile_h == best_c.lap_tile_h && c.bil_tile_h == best_c.bil_tile_h) continue;   // timed
+                round2.push_back(c);
             }
         try_all(round2);
     }
