@@ -177,7 +177,7 @@ __device__ __forceinline__ float lap_scale(bool keep, float lambda, float ws) {
 
 // Top-left element (x0, u0) of a Laplacian tile's box in the AoS array seen as H rows of 3W
 // floats, and the offset of the tile's first point inside its box row. Tiles are th points high
-// (th = 32, or 64 for a single-iteration first pass) and T = 32 points wide.
+// (LapPhase::tile_h, 16 to 64) and T = 32 points wide.
 struct LapOrigin {
     int u0, c0, x0, dlt;
 };
@@ -240,8 +240,8 @@ __device__ __forceinline__ void lap_issue(const FrameArgs& a, const LapPhase& ph
 // tile: from `cur` (displacements; unused when WITH_D = false) into `nxt`. Each thread walks down
 // one column of a segment of rows with a three-row window in registers: a row costs the loads of
 // three points, and its S edge is the next row's N edge. What bounds the pass is instruction issue
-// and the barrier after each iteration; the segments are cut so that every thread gets the same
-// number of rows (7, 6, 6, 5, 4 in five iterations of a 32 x 32 tile), where strips of four rows took
+// and the barrier after each iteration; the segments are cut as evenly as whole rows allow (at most
+// 7, 7, 6, 5, 4 rows a thread in five iterations of a 32 x 32 tile), where strips of four rows took
 // two rounds of the CTA for four of the five: 256 mixed frames 5723 -> 5656 us, 720x1280 181.6 ->
 // 179.8 us.
 // Every point takes its window in row-major order, so its sum does not depend on where the segments
@@ -665,7 +665,8 @@ __device__ __forceinline__ V3 own_sum(const OwnTri& o) {
 // A quad's two triangles: their own quad first. Each triangle's weight with itself is exactly 1, so what
 // is left is one weight of each with the other, in scalar steps that share the difference of the
 // centroids (the same roundings as a half of own_weights): 21 FP32 cycles instead of 48 of a quad's 432,
-// a packed instruction taking two. 480x640 frame 64.4 -> 64.0 us, 256 frames 5012 -> 4969 us.
+// a packed instruction taking two. 480x640 frame 64.4 -> 64.0 us. In the batch kernel the iterations' own
+// CTA time rose with it (256 frames 383 -> 391 ms) while the bilateral phase took 3392 -> 3364 us.
 struct QuadAcc {
     OwnTri t0, t1;
     V3 n0, n1;   // current normals (a triangle without a normal keeps n = 0)
@@ -1462,7 +1463,8 @@ __device__ __forceinline__ void merge_phase(const FrameArgs& a) {
 // bytes per lane. With both, the phase took 0.38 ms and the batch 5.88 instead of 7.40 ms; a 480x640
 // frame 69.6 instead of 73.7 us. After that a warp waits for one load after another, so a batch,
 // whose warps take dozens of blocks each, has kFlatVecBatch loads per lane in flight (417 us at 2, 278 us
-// at 4, 178 us at 8); a single frame has less than a block per warp, and 4 cost it 0.9 us.
+// at 4, 178 us at 8); a 480x640 frame has less than a block per warp, and 4 cost it 0.9 us (a 720x1280 frame
+// has three, at 2 as well).
 constexpr int kFlatVec = 2, kFlatVecBatch = 8;
 template <int VEC>
 constexpr int kFlatBlock = 32 * 4 * VEC;

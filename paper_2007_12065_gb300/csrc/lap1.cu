@@ -20,7 +20,7 @@
 // diagonals inside the pair (SE of the left point and SW of the right one become NW and NE of the
 // next row's pair). Only the weight of a shared diagonal is kept; its difference is formed again.
 //
-// Every point is the same arithmetic as in lap_iteration (frame_kernels.cuh): its window in
+// Every point is the same arithmetic as in lap_walk (frame_kernels.cuh): its window in
 // row-major order (NW, N, NE, W, E, SW, S, SE), a shared edge entering with its difference negated
 // (w_ij = w_ji, opposite differences), the same rounding intrinsics. Passes of this kernel and fused
 // tile passes therefore give the same bits, and a batch the same bits as single frames.

@@ -25,8 +25,9 @@ constexpr int kThreads = 256;    // threads per CTA
 constexpr int kTile = 32;        // tile edge: 32 x 32 points (Laplacian) or quads (bilateral)
 constexpr int kLapMaxHalo = 8;   // largest halo (fused iterations x radius) of one Laplacian pass
 constexpr int kBilMaxHalo = 6;   // same for the bilateral
-// Shared memory per CTA that still lets two CTAs share an SM (the bilateral pass at halo 3 needs
-// this much); a Laplacian pass stages as many boxes ahead as fit within it.
+// Shared memory per CTA up to which two CTAs share an SM (half of its 228 KB, less 1 KB per CTA, is
+// 115,712 bytes; the bilateral pass at halo 3 needs 113,872); a Laplacian pass stages as many boxes
+// ahead as fit within it.
 constexpr int kTwoCtaSmem = 114048;
 constexpr int kLapMaxStages = 3;   // box buffers of a Laplacian pass: this tile's and up to 2 ahead
 constexpr int kLapThinTileH = 64;  // tile height of a single-iteration first Laplacian pass
@@ -241,9 +242,9 @@ struct Tuning {
     int bil_fuse;                  // same for the bilateral
     int ctas_per_sm;               // 0 = as many as fit
     int lap_tile_h;                // Laplacian tile height in points, 0 = by frame_tuning for a single
-                                   // frame, 32 in a batch (64 with a 3 x 3 window and for a
-                                   // single-iteration first pass); a
-                                   // height whose buffers would not fit two CTAs per SM falls back to 32
+                                   // frame, 64 for a single-iteration first pass, else 32 (a batch
+                                   // with a 3 x 3 window asks for 64); a height whose buffers would
+                                   // not fit two CTAs per SM falls back to 32
     int bil_tile_h;                // bilateral tile height in quads, 0 = by frame_tuning for a single
                                    // frame, 32 in a batch
 };
