@@ -190,13 +190,15 @@ static double phase_cost(long long tiles, int sms, int per_sm, bool crowded, dou
 
 // Tile heights of a single frame whose tuning leaves them open. A phase lasts as long as its
 // rounds of tiles, and a tile's time is a fixed part plus a part per row, so low tiles win where 32
-// rows would leave SMs idle (a 120x160 frame has 20 such tiles for 304 CTAs: 49.7 us at 32 rows,
-// 36.1 us at 8-row bilateral tiles) or start one more round for a few tiles (720x1280: 920 tiles at
-// 32 rows, 1,200 at 24; 224 and 201 us), and tall ones where they save a round (its Laplacian at 48
-// rows: 224 and 206 us). The times below, in us, are a fit to such sweeps on a GB300 (2.07 GHz):
-// staging and geometry per staged row, iterations per row and iteration, groups and labels per
-// row; a tile alone on its SM takes 0.66 (bilateral) or 0.8
-// (Laplacian) of the time of each of two.
+// rows would leave SMs idle (a 120x160 frame has 20 such tiles for 304 CTAs: 45.1 us at 32 rows,
+// 34.4 us at 8-row bilateral tiles, 30.8 us with 16-row Laplacian tiles too) or start one more round for a
+// few tiles (720x1280: 920 tiles at 32 rows, 1,200 at 24; 213.6 and 190.7 us), and tall ones where they
+// save a round (its Laplacian at 48 rows: 213.6 and 193.9 us). The times below, in us, are a fit to
+// sweeps on a GB300 (2.07 GHz) of an earlier state of these kernels: staging and geometry per staged
+// row, iterations per row and iteration, groups and labels per row; a tile alone on its SM takes 0.66
+// (bilateral) or 0.8 (Laplacian) of the time of each of two. With the present kernels the chosen pair
+// takes at most 1.05 times the best of 24 pairs on 26 frames of 12 thousand to 0.9 million points, and
+// at most 1.02 times 32 rows for both.
 //
 // Both phases run on one grid, that of the phase with more tiles, so the two heights are chosen
 // together: 228 Laplacian tiles of 16 rows put two CTAs on some SMs, and 114 bilateral tiles then take
